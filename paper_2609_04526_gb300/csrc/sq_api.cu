@@ -250,10 +250,57 @@ void free_scratch(Scratch &s) {
   s.retired.clear();
 }
 
+// One forward or input gradient on the few-token kernel. tiles: the device list of a
+// grouped call's token tiles, or null (equal tiles of tile_tokens over M).
+sq_status run_few(sq_handle h, DeviceState *dev, int mode, int fmt, int E, int64_t N, int64_t K, const uint8_t *codes,
+                  const uint8_t *scales, float ws2, const void *a_ptr, int64_t M, void *out, const sqi::FewTile *tiles,
+                  int64_t token_tiles, int tile_tokens, cudaStream_t stream) {
+  CUtensorMap tmX[3];
+  const int64_t inner = mode == sqi::MODE_FWD ? K : N;
+  if (tiles) {
+    for (int i = 0; i < 3; ++i) SQ_TRY(make_act_map(h, &tmX[i], a_ptr, inner, M, 64, sqi::kFewBoxRows << i));
+  } else {
+    SQ_TRY(make_act_map(h, &tmX[0], a_ptr, inner, M, 64, sqi::few_box_rows(tile_tokens)));
+    tmX[1] = tmX[2] = tmX[0];
+  }
+  CUtensorMap tmCodes;  // all experts' codes as one [E * N, K/2] tensor
+  SQ_TRY(make_map(h, &tmCodes, codes, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, K / 2, E * N, 64, 128,
+                  CU_TENSOR_MAP_SWIZZLE_64B));
+  sqi::FewArgs f;
+  f.mode = mode;
+  f.fmt = fmt;
+  f.M = M;
+  f.N = N;
+  f.K = K;
+  f.scales = scales;
+  f.ws2 = ws2;
+  f.out = static_cast<uint16_t *>(out);
+  f.err = dev->err_word;
+  f.tiles = tiles;
+  f.tile_tokens = tile_tokens;
+  f.units = token_tiles * (((mode == sqi::MODE_FWD ? N : K) + sqi::kFewFeatures - 1) / sqi::kFewFeatures);
+  const cudaError_t e = sqi::launch_few(f, tmX, tmCodes, dev->sm_count, stream);
+  if (e != cudaSuccess) return cuda_fail(h, e, "few-token kernel launch");
+  return SQ_OK;
+}
+
 sq_status run_gemm(sq_handle h, int mode, const sq_weight *w, const void *a_ptr, const void *b_ptr, int64_t M,
                    void *out, const uint8_t *mask, cudaStream_t stream) {
   DeviceState *dev = nullptr;
   SQ_TRY(ensure_device(h, &dev));
+  if (mode != sqi::MODE_SGRAD) {
+    const int64_t F = mode == sqi::MODE_FWD ? w->N : w->K, Kc = mode == sqi::MODE_FWD ? w->K : w->N;
+    const int64_t pair_tiles =
+        ((M + sqi::kPairMTile - 1) / sqi::kPairMTile) * ((F + sqi::kPairNTile - 1) / sqi::kPairNTile);
+    auto tiles_at = [&](int limit) {
+      const int t = sqi::few_tile_tokens(M, limit);
+      return (M + t - 1) / t;
+    };
+    const int limit = sqi::few_limit(tiles_at, M, F, Kc, pair_tiles, dev->sm_count);
+    if (limit > 0)
+      return run_few(h, dev, mode, w->fmt, 1, w->N, w->K, w->codes, w->scales, w->ws2, a_ptr, M, out, nullptr,
+                     tiles_at(limit), sqi::few_tile_tokens(M, limit), stream);
+  }
   CUtensorMap tmA, tmB, tmOut;
   const int64_t K2 = w->K / 2;  // code bytes per row
   if (mode == sqi::MODE_FWD) {
@@ -473,6 +520,46 @@ sq_status run_grouped(sq_handle h, int mode, const sq_grouped_weight *w, const s
   }
   tile_start[E] = static_cast<int32_t>(total);
   if (total == 0) return SQ_OK;
+
+  if (mode != sqi::MODE_SGRAD) {
+    const int64_t F = mode == sqi::MODE_FWD ? N : K, Kc = mode == sqi::MODE_FWD ? K : N;
+    auto tiles_at = [&](int limit) {
+      int64_t tiles = 0;
+      for (int x = 0; x < E; ++x)
+        if (rows[x] > 0) {
+          const int t = sqi::few_tile_tokens(rows[x], limit);
+          tiles += (rows[x] + t - 1) / t;
+        }
+      return tiles;
+    };
+    const int limit = sqi::few_limit(tiles_at, offsets[E], F, Kc, total, dev->sm_count);
+    if (limit > 0) {
+      const int64_t token_tiles = tiles_at(limit);
+      int tokens = 0;  // of the largest token tile
+      for (int x = 0; x < E; ++x)
+        if (rows[x] > 0) tokens = std::max(tokens, sqi::few_tile_tokens(rows[x], limit));
+      TableSlot *t = nullptr;
+      const size_t bytes = static_cast<size_t>(token_tiles) * sizeof(sqi::FewTile);
+      SQ_TRY(acquire_table(h, dev, bytes, &t));
+      auto *list = reinterpret_cast<sqi::FewTile *>(t->host);
+      for (int x = 0; x < E; ++x) {
+        if (rows[x] == 0) continue;
+        const int64_t step = sqi::few_tile_tokens(rows[x], limit);
+        for (int64_t r = 0; r < rows[x]; r += step)
+          *list++ = {x, static_cast<int>(offsets[x] + r), static_cast<int>(std::min(step, rows[x] - r)),
+                     w->ws2 ? w->ws2[x] : 1.0f};
+      }
+      if ((e = cudaMemcpyAsync(t->dev, t->host, bytes, cudaMemcpyHostToDevice, stream)) != cudaSuccess)
+        return cuda_fail(h, e, "copying the token tiles");
+      const sq_status st = run_few(h, dev, mode, w->fmt, E, N, K, w->codes, w->scales, 1.0f, a_ptr, offsets[E], out,
+                                   reinterpret_cast<const sqi::FewTile *>(t->dev), token_tiles, tokens, stream);
+      const cudaError_t e2 = cudaEventRecord(t->done, stream);
+      if (e2 == cudaSuccess) t->pending = true;
+      if (st != SQ_OK) return st;
+      if (e2 != cudaSuccess) return cuda_fail(h, e2, "cudaEventRecord(table)");
+      return SQ_OK;
+    }
+  }
 
   TableSlot *t = nullptr;
   const size_t bytes = sqi::group_table_bytes(E);

@@ -89,6 +89,121 @@ inline int sgrad_splits(int64_t tiles, int clusters, int64_t M) {
   return 1;
 }
 
+// Forward / input gradient over few tokens (sq_few.cu): tiles of kFewFeatures output
+// features x up to kFewTokens tokens. A grouped call lists its token tiles in device
+// memory (an expert's rows cut into equal tiles); a CTA takes a token tile and a feature
+// tile.
+constexpr int kFewFeatures = 128;
+constexpr int kFewTokens = 256;        // of a tile, where every CTA has an SM alone
+constexpr int kFewTokensShared = 192;  // ... where two CTAs share an SM
+constexpr int kFewBoxRows = 32;        // tokens of the smallest TMA box
+constexpr int kFewSmemBytes = 111 * 1024;  // of a CTA: two share an SM
+constexpr int kFewSmemAlone = 224 * 1024;  // ... where the launch has at most one CTA per SM
+constexpr int kFewSlotBytes = 128 * 64;    // packed codes of 128 x 128 weights
+constexpr int kFewMaxStages = 4, kFewMaxSlots = 12;
+
+// Tokens of the equal tiles (whole MMA steps of 16) that `rows` tokens are cut into.
+inline int few_tile_tokens(int64_t rows, int limit) {
+  const int64_t tiles = (rows + limit - 1) / limit;
+  return static_cast<int>(((rows + tiles - 1) / tiles + 15) / 16 * 16);
+}
+// Token rows of a stage's activations: whole boxes.
+inline int few_box_rows(int tile_tokens) {
+  return (tile_tokens + kFewBoxRows - 1) / kFewBoxRows * kFewBoxRows;
+}
+
+// Shared memory of a CTA: `stages` stages of `depth` contraction indices (decoded weights
+// and activations) and `slots` code slots, so the codes run ahead of the MMAs by the slots
+// less the stages' share of them. The epilogue's bf16 tile reuses the stages.
+struct FewRing {
+  int depth, stage_bytes, stages, slots;
+  int bytes;  // with 1 KiB for the alignment
+};
+inline FewRing few_ring(int tile_tokens, bool alone) {
+  FewRing r;
+  const int rows = few_box_rows(tile_tokens);
+  const int room = (alone ? kFewSmemAlone : kFewSmemBytes) - 1024;
+  r.depth = alone ? 128 : 64;
+  r.stage_bytes = (kFewFeatures + rows) * r.depth * 2;
+  if (alone)
+    r.stages = rows <= 96 ? 3 : 2;
+  else
+    r.stages = rows <= 32 ? 4 : rows <= 64 ? 3 : 2;
+  r.slots = (room - r.stages * r.stage_bytes) / kFewSlotBytes;
+  if (r.slots > kFewMaxSlots) r.slots = kFewMaxSlots;
+  r.bytes = r.stages * r.stage_bytes + r.slots * kFewSlotBytes + 1024;
+  return r;
+}
+
+struct FewTile {
+  int expert, row0, rows;
+  float ws2;
+};
+struct FewArgs {
+  int mode, fmt;
+  int64_t M, N, K;
+  const uint8_t *scales;
+  float ws2;
+  uint16_t *out;
+  int *err;
+  const FewTile *tiles;  // device list of a grouped call, or null: tiles of tile_tokens over M
+  int tile_tokens;       // tokens of the largest tile (<= kFewTokens)
+  int64_t units;
+};
+// Which kernel runs a forward or input gradient, by estimates of both in microseconds that
+// were fitted to measured launches (weights of 4096 x 4096, 1024 x 4096, 14336 x 4096, 768 x
+// 2048 and 256 x 512 at 16 to 4096 tokens; 128 experts of 768 x 2048 and 2880 x 2880 with 2 to
+// 1024 rows each) and lie within 20 % of them above 15 us. Both sides of the line, few-token
+// against pair kernel, in us: 4096 x 4096 25 against 43 at 16 to 512 tokens, 31 against 45 at
+// 1024, 78 against 45 at 2048; 1024 x 4096 25 against 44 at 2048; 768 x 2048 experts 77 against
+// 127 with 64 rows each, 139 against 148 with 256, 223 against 198 with 512; 2880 x 2880
+// experts 271 against 566 with 16 rows each, 345 against 520 with 128, 581 against 567 with 256.
+//
+// few_us, for token tiles of `tokens` tokens on average: a CTA alone on its SM takes 0.61 us
+// per 128-deep stage, more above 128 tokens (two stages in flight); CTAs that share an SM 0.27
+// us and up with the tokens per 64-deep stage, and 1.5 us to start and drain.
+inline double few_us(int64_t token_tiles, double tokens, int64_t features, int64_t contraction, int sm_count) {
+  const int64_t ctas = token_tiles * ((features + kFewFeatures - 1) / kFewFeatures);
+  if (ctas <= sm_count)
+    return 4.8 + ((contraction + 127) / 128) * (0.61 + (tokens > 128 ? 0.0015 * (tokens - 128) : 0.0));
+  const double per_sm = ctas > 4 * sm_count ? static_cast<double>(ctas) / sm_count
+                                            : static_cast<double>((ctas + sm_count - 1) / sm_count);
+  return 4.8 + per_sm * (((contraction + 63) / 64) * (0.27 + 0.0006 * tokens) + 1.5);
+}
+// A wave of 512 x 256 pair tiles lasts 1.08 us per 128-deep k-step and 4 us at its end.
+inline double pair_us(int64_t tiles, int64_t contraction, int sm_count) {
+  const int64_t clusters = sm_count / 2, waves = (tiles + clusters - 1) / clusters;
+  return 9.5 + waves * (1.08 * ((contraction + 127) / 128)) + 4.0 * (waves - 1);
+}
+// The limit of a token tile (few_tile_tokens) of the few-token launch over `rows` tokens in
+// all, or 0 where the pair kernel's `pair_tiles` tiles are the faster launch. `tiles_at`
+// counts the token tiles at a limit.
+template <class TilesAt>
+inline int few_limit(TilesAt tiles_at, int64_t rows, int64_t features, int64_t contraction, int64_t pair_tiles,
+                     int sm_count) {
+  if (sm_count < 2) return 0;
+  double best_us = 0.97 * pair_us(pair_tiles, contraction, sm_count);
+  int best = 0;
+  for (int limit : {kFewTokens / 2, kFewTokensShared, kFewTokens}) {
+    const int64_t tiles = tiles_at(limit);
+    const int64_t ctas = tiles * ((features + kFewFeatures - 1) / kFewFeatures);
+    if (ctas > (int64_t(1) << 24) || (limit > kFewTokensShared && ctas > sm_count)) continue;
+    const double us = few_us(tiles, static_cast<double>(rows) / tiles, features, contraction, sm_count);
+    if (us < best_us) {
+      best_us = us;
+      best = limit;
+    }
+  }
+  return best;
+}
+
+// tmX: the activations [M, contraction] in boxes of 64 x kFewBoxRows, 2 kFewBoxRows
+// and 4 kFewBoxRows (a dense launch: the first in boxes of 64 x few_box_rows), 128-byte
+// swizzle; tmCodes: the packed codes in boxes of 64 bytes x 128
+// rows, 64-byte swizzle.
+cudaError_t launch_few(const FewArgs &a, const CUtensorMap (&tmX)[3], const CUtensorMap &tmCodes, int sm_count,
+                       cudaStream_t stream);
+
 struct GroupedArgs {
   int mode;
   int fmt;
