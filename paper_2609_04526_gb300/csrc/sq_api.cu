@@ -1000,7 +1000,7 @@ sq_status sq_project_lowrank(sq_handle h, int32_t fmt, int64_t N, int64_t G, int
   if (mask_out && !aligned16(mask_out)) return fail(h, SQ_ERR_INVALID_ARG, "mask_out must be 16-byte aligned");
   if (latent_out && !aligned16(latent_out)) return fail(h, SQ_ERR_INVALID_ARG, "latent_out must be 16-byte aligned");
   e = sqi::launch_project_lowrank(fmt, N, G, r, ws2, alpha_over_r, base_scales, B, A, bytes_out, mask_out, nonfinite,
-                                  latent_out, st);
+                                  latent_out, dev->sm_count, st);
   if (e != cudaSuccess) return cuda_fail(h, e, "adapter projection launch");
   return SQ_OK;
   SQ_GUARD_END
@@ -1265,7 +1265,7 @@ sq_status sq_grouped_project_lowrank(sq_handle h, const sq_grouped_weight *w, in
   cudaError_t e;
   if (w->fmt == SQ_MXFP4) {
     e = sqi::launch_project_lowrank(w->fmt, N, G, r, 1.0f, alpha_over_r, w->scales, B, A, bytes_out, mask_out,
-                                    nonfinite, latent_out, st, w->E, nullptr);
+                                    nonfinite, latent_out, dev->sm_count, st, w->E, nullptr);
     if (e != cudaSuccess) return cuda_fail(h, e, "grouped adapter projection launch");
     return SQ_OK;
   }
@@ -1276,7 +1276,7 @@ sq_status sq_grouped_project_lowrank(sq_handle h, const sq_grouped_weight *w, in
   if ((e = cudaMemcpyAsync(t->dev, t->host, tbytes, cudaMemcpyHostToDevice, st)) != cudaSuccess)
     return cuda_fail(h, e, "copying the expert tensor scales");
   e = sqi::launch_project_lowrank(w->fmt, N, G, r, 1.0f, alpha_over_r, w->scales, B, A, bytes_out, mask_out,
-                                  nonfinite, latent_out, st, w->E, reinterpret_cast<const float *>(t->dev));
+                                  nonfinite, latent_out, dev->sm_count, st, w->E, reinterpret_cast<const float *>(t->dev));
   cudaError_t e2 = cudaEventRecord(t->done, st);
   if (e2 == cudaSuccess) t->pending = true;
   if (e != cudaSuccess) return cuda_fail(h, e, "grouped adapter projection launch");

@@ -292,8 +292,8 @@ cudaError_t launch_swap_or_diff(int64_t count, const uint8_t *a, uint8_t *b, boo
 // launch for all); ws2_per (device, NVFP4) gives each expert's tensor scale.
 cudaError_t launch_project_lowrank(int fmt, int64_t N, int64_t G, int r, float ws2, float alpha_over_r,
                                    const uint8_t *base, const uint16_t *B, const uint16_t *A, uint8_t *bytes_out,
-                                   uint8_t *mask_out, int32_t *nonfinite, float *latent_out, cudaStream_t stream,
-                                   int experts = 1, const float *ws2_per = nullptr);
+                                   uint8_t *mask_out, int32_t *nonfinite, float *latent_out, int sm_count,
+                                   cudaStream_t stream, int experts = 1, const float *ws2_per = nullptr);
 // Ranks up to 128 run on the tensor cores (sq_adapter_tc.cu), larger ones on CUDA
 // cores; `err` is the device error word (bounded waits of the tensor-core path).
 size_t lowrank_grad_workspace(int64_t N, int64_t G, int r, int sm_count, int experts = 1);

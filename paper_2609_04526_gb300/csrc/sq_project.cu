@@ -28,6 +28,69 @@ __device__ __forceinline__ uint32_t e4m3x2_rn(float lo, float hi) {
   return r;
 }
 
+// Packed fp32 pairs: both halves of an operation are rounded by themselves.
+__device__ __forceinline__ uint64_t fma_x2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+
+__device__ __forceinline__ uint64_t dup_x2(float v) {
+  uint64_t d;
+  asm("mov.b64 %0, {%1, %1};" : "=l"(d) : "f"(v));
+  return d;
+}
+__device__ __forceinline__ uint64_t mul_x2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ uint64_t pair_x2(float lo, float hi) {
+  uint64_t d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
+  return d;
+}
+__device__ __forceinline__ float lo_x2(uint64_t a) { return __uint_as_float(static_cast<uint32_t>(a)); }
+__device__ __forceinline__ float hi_x2(uint64_t a) { return __uint_as_float(static_cast<uint32_t>(a >> 32)); }
+
+// Quotients a/b by a plane's tensor scale b that round to the same E4M3 byte as the
+// correctly rounded fp32 quotient: q = a y with y = 1/b rounded to nearest, then one
+// correction q + (a - b q) y (the step of Markstein's division, "Computation of elementary
+// functions on the IBM RISC System/6000 processor", 1990), three packed instructions for
+// two latents against ~15 for each of a general division. The remainder is exact, so the
+// corrected value is the rounding of a/b + d with |d| <= 3 * 2^-25 ulp. It can differ from
+// the rounding of a/b only where a/b lies within d of the middle of two floats, and the byte
+// only where one of the two is a rounding point m of the grid: a/b = m + (1/2 + e) ulp,
+// 0 < |e| <= |d|. With the 24-bit integers M and B of m and b, (2 M + 1) B + 2 e B is then a
+// multiple of 2^24, and M, five significant bits, one of 2^19: so B +- k is a multiple of
+// 2^20 for a k = 2 |e| B in {1, 2, 3}. Tensor scales with such a B take the general
+// division, and so do those outside [2^-90, 2^90], where the remainder could underflow;
+// inside, a quotient too small for a nonzero byte keeps its sign. The products are formed
+// for -a, which gives both zeros their own sign.
+struct TensorScale {
+  float b, cap;
+  bool plain;  // general division
+  uint64_t b2, ny2;
+  __device__ __forceinline__ TensorScale(float ws2, float cap_) {
+    b = ws2;
+    cap = cap_;
+    const uint32_t low = ((__float_as_uint(ws2) & 0xFFFFFu) + 3u) & 0xFFFFFu;  // B + 3 mod 2^20
+    plain = !(ws2 >= 0x1p-90f && ws2 <= 0x1p90f) || (low <= 6u && low != 3u);
+    b2 = dup_x2(ws2);
+    ny2 = dup_x2(-__frcp_rn(ws2));
+  }
+  __device__ __forceinline__ uint64_t negated_quotients(uint64_t a) const {
+    const uint64_t q = mul_x2(a, ny2);
+    return fma_x2(fma_x2(q, b2, a), ny2, q);
+  }
+};
+
+__device__ __forceinline__ float max_nan(float a, float b) {  // NaN if either is
+  float r;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
+
 // NVFP4 projection of one latent (absolute units) to (byte, mask, is_nan).
 __device__ __forceinline__ void project_nv(float L, float ws2, float cap, uint32_t &byte, uint32_t &mask,
                                            uint32_t &nan) {
@@ -105,6 +168,24 @@ __device__ __forceinline__ float scale_value(uint32_t byte, float ws2) {
   return __uint_as_float(byte << 23);
 }
 
+// The four on-grid scales of four consecutive bytes, each exactly as scale_value.
+template <int FMT>
+__device__ __forceinline__ void scale_value4(uint32_t bytes, float ws2, float (&s)[4]) {
+  if (FMT == 0) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      uint32_t hf;
+      asm("cvt.rn.f16x2.e4m3x2 %0, %1;" : "=r"(hf) : "h"(static_cast<unsigned short>(bytes >> (16 * h))));
+      const __half2 v = *reinterpret_cast<const __half2 *>(&hf);
+      s[2 * h] = __fmul_rn(__low2float(v), ws2);
+      s[2 * h + 1] = __fmul_rn(__high2float(v), ws2);
+    }
+  } else {
+#pragma unroll
+    for (int c = 0; c < 4; ++c) s[c] = scale_value<FMT>((bytes >> (8 * c)) & 0xFFu, ws2);
+  }
+}
+
 __device__ __forceinline__ void warp_add_i32(int32_t *counter, uint32_t v) {
   v = __reduce_add_sync(0xFFFFFFFFu, v);
   if ((threadIdx.x & 31) == 0 && v) atomicAdd(counter, static_cast<int32_t>(v));
@@ -114,6 +195,62 @@ __device__ __forceinline__ void warp_add_i64(int64_t *counter, uint32_t v) {
   v = __reduce_add_sync(0xFFFFFFFFu, v);
   if ((threadIdx.x & 31) == 0 && v)
     atomicAdd(reinterpret_cast<unsigned long long *>(counter), static_cast<unsigned long long>(v));
+}
+
+// Four consecutive blocks of a plane (one float4 of latents) -> their bytes, mask bytes
+// and NaN count, each block exactly as project_one. One maximum, NaN if any latent is,
+// tells whether there is anything to clamp or count, and NVFP4 converts two blocks per
+// instruction; MXFP4's rounding of a normal latent's exponent is one integer addition,
+// whose carry out of the significand is the test against sqrt(2).
+template <int FMT>
+__device__ __forceinline__ void project4(float4 L4, const TensorScale &ts, uint32_t &bytes, uint32_t &mask,
+                                         uint32_t &nan) {
+  const float l[4] = {L4.x, L4.y, L4.z, L4.w};
+  if (FMT == 0) {
+    const float top = max_nan(max_nan(fabsf(l[0]), fabsf(l[1])), max_nan(fabsf(l[2]), fabsf(l[3])));
+    if (top == top && !ts.plain) {
+      float c[4] = {l[0], l[1], l[2], l[3]};
+      mask = 0x01010101u;
+      if (top > ts.cap) {
+        mask = 0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          mask |= (fabsf(l[i]) <= ts.cap ? 1u : 0u) << (8 * i);
+          c[i] = fminf(fmaxf(l[i], -ts.cap), ts.cap);
+        }
+      }
+      const uint64_t q0 = ts.negated_quotients(pair_x2(c[0], c[1])), q1 = ts.negated_quotients(pair_x2(c[2], c[3]));
+      bytes = (e4m3x2_rn(lo_x2(q0), hi_x2(q0)) | (e4m3x2_rn(lo_x2(q1), hi_x2(q1)) << 16)) ^ 0x80808080u;
+      nan = 0;
+      return;
+    }
+  } else {
+    constexpr uint32_t kFirst = 0x00800000u;            // 2^-126
+    constexpr uint32_t kSpan = 0x7F3504F4u - kFirst;    // to the last value that rounds to 2^127
+    uint32_t u[4], far = 0;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      u[c] = __float_as_uint(l[c]);
+      far = max(far, u[c] - kFirst);  // also large for negative values, zeros, subnormals, inf and NaN
+    }
+    if (far < kSpan) {
+#pragma unroll
+      for (int c = 0; c < 4; ++c) u[c] = (u[c] + (0x00800000u - 0x003504F4u)) >> 23;
+      bytes = u[0] | (u[1] << 8) | (u[2] << 16) | (u[3] << 24);
+      mask = 0x01010101u;
+      nan = 0;
+      return;
+    }
+  }
+  bytes = mask = nan = 0;
+#pragma unroll 1
+  for (int c = 0; c < 4; ++c) {  // rare: rolled up, to keep the callers small
+    uint32_t b, m, n;
+    project_one<FMT>(c == 0 ? l[0] : c == 1 ? l[1] : c == 2 ? l[2] : l[3], ts.b, ts.cap, b, m, n);
+    bytes |= b << (8 * c);
+    mask |= m << (8 * c);
+    nan += n;
+  }
 }
 
 // Planes of several experts in one launch (PER instantiations): element i belongs
@@ -234,17 +371,21 @@ __global__ void __launch_bounds__(kThreads) sq_merge_kernel(int64_t count, float
 //
 // The planes of all linears of a layer (Sec. 5 Payoff 3: the merge touches every
 // target linear) in one launch each for projection and merge. Every CTA works on
-// kPlaneVecs 16-element vectors of one plane (the CTAs of plane j follow those of
-// plane j - 1), so it reduces its counter within the block and adds it with one
+// kThreads x kProjectF4 (kMergeF4) float4s of one plane's latents (the CTAs of plane j
+// follow those of plane j - 1), so it reduces its counter within the block and adds it with one
 // atomic; the last CTA to finish (a ticket) writes every plane's count and clears
 // the accumulators for the next call.
-constexpr int kPlaneVecsPerThread = 2;
-constexpr int kPlaneVecs = kThreads * kPlaneVecsPerThread;
+constexpr int kProjectF4 = 8, kMergeF4 = 4;  // float4s of latents per thread
 
+__host__ __device__ __forceinline__ int64_t plane_ctas(int64_t count, int f4) {
+  return (count / 4 + kThreads * f4 - 1) / (kThreads * f4);
+}
+
+template <int F4>
 __device__ __forceinline__ int plane_of_block(const PlaneTable &t, int64_t b, int64_t &first_block) {
   int64_t start = 0;
   for (int j = 0; j < t.n; ++j) {
-    const int64_t nb = (t.p[j].count / 16 + kPlaneVecs - 1) / kPlaneVecs;
+    const int64_t nb = plane_ctas(t.p[j].count, F4);
     if (b < start + nb) {
       first_block = start;
       return j;
@@ -290,72 +431,39 @@ __device__ __forceinline__ void plane_counters(const PlaneTable &t, int j, uint3
   *ticket = 0u;
 }
 
-// Four consecutive blocks of a plane (one float4 of latents) -> their bytes, mask bytes
-// and NaN count, each block exactly as project_one. NVFP4 converts two blocks per
-// instruction; a NaN latent's byte is patched afterwards (rare).
+// Lane t of the CTA takes float4 t + kThreads * i of its chunk, so each warp-wide load
+// reads 512 contiguous bytes and each store of bytes writes 128. A thread loads all its
+// latents (and, merging, the old bytes) before it computes and stores any: the byte stores
+// could alias the latent loads as far as the compiler knows, so interleaving them would
+// serialise every float4 on the memory latency. Bound by the memory system at these sizes:
+// the 82 MB of the 8B layer's NVFP4 planes take 21 us projected and 19 us merged (before
+// project4's short paths 23 and 21), the 41 MB of its MXFP4 planes 12.6 and 12.1 us (18.2 and
+// 17.8). The merge, with the old bytes to hold, is faster with half the float4s per thread;
+// one wave of CTAs that walk the chunks, the next chunk's loads in flight, took 2-3 us more.
 template <int FMT>
-__device__ __forceinline__ void project4(float4 L4, float ws2, float cap, uint32_t &bytes, uint32_t &mask,
-                                         uint32_t &nan) {
-  const float l[4] = {L4.x, L4.y, L4.z, L4.w};
-  bytes = mask = nan = 0;
-  if (FMT == 0) {
-    float q[4];
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      nan += (l[c] != l[c]) ? 1u : 0u;
-      mask |= (fabsf(l[c]) <= cap ? 1u : 0u) << (8 * c);  // false for NaN, as -cap <= L <= cap
-      q[c] = __fdiv_rn(fminf(fmaxf(l[c], -cap), cap), ws2);
-    }
-    bytes = e4m3x2_rn(q[0], q[1]) | (e4m3x2_rn(q[2], q[3]) << 16);
-    if (nan) {
-#pragma unroll
-      for (int c = 0; c < 4; ++c)
-        if (l[c] != l[c]) bytes = (bytes & ~(0xFFu << (8 * c))) | (0x7Fu << (8 * c));
-    }
-  } else {
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      uint32_t b, m, n;
-      project_one<FMT>(l[c], ws2, cap, b, m, n);
-      bytes |= b << (8 * c);
-      mask |= m << (8 * c);
-      nan += n;
-    }
-  }
-}
-
-// A CTA's chunk is kPlaneVecs x 16 blocks: lane t of the CTA takes float4 t + kThreads * i
-// of it (i < 4 kPlaneVecsPerThread), so each warp-wide load reads 512 contiguous bytes and
-// each store of bytes writes 128. A thread loads all its latents (and, merging, the old
-// bytes) before it computes and stores any: the byte stores could alias the latent
-// loads as far as the compiler knows, so interleaving them would serialise every
-// float4 on the memory latency.
-constexpr int kPlaneF4 = 4 * kPlaneVecsPerThread;  // float4s per thread per chunk
-
-template <int FMT>
-__global__ void __launch_bounds__(kThreads) sq_project_planes_kernel(const __grid_constant__ PlaneTable t,
+__global__ void __launch_bounds__(kThreads, 5) sq_project_planes_kernel(const __grid_constant__ PlaneTable t,
                                                                         int64_t *acc) {
   __shared__ uint32_t red[kThreads / 32];
   int64_t first_block;
-  const int j = plane_of_block(t, blockIdx.x, first_block);
+  const int j = plane_of_block<kProjectF4>(t, blockIdx.x, first_block);
   const PlaneArgs &pl = t.p[j];
-  const float ws2 = pl.ws2, cap = 448.0f * pl.ws2;  // the same IEEE fp32 product as the single-plane cap
+  const TensorScale ts(pl.ws2, 448.0f * pl.ws2);  // the same IEEE fp32 product as the single-plane cap
   const int64_t nf4 = pl.count / 4;
-  const int64_t f0 = (static_cast<int64_t>(blockIdx.x) - first_block) * (4 * kPlaneVecs) + threadIdx.x;
+  const int64_t f0 = (static_cast<int64_t>(blockIdx.x) - first_block) * (kThreads * kProjectF4) + threadIdx.x;
   const float4 *src = reinterpret_cast<const float4 *>(pl.latent);
-  float4 L[kPlaneF4];
+  float4 L[kProjectF4];
 #pragma unroll
-  for (int i = 0; i < kPlaneF4; ++i) {
+  for (int i = 0; i < kProjectF4; ++i) {
     const int64_t f = f0 + static_cast<int64_t>(i) * kThreads;
     if (f < nf4) L[i] = __ldcs(src + f);
   }
   uint32_t nan_count = 0;
 #pragma unroll
-  for (int i = 0; i < kPlaneF4; ++i) {
+  for (int i = 0; i < kProjectF4; ++i) {
     const int64_t f = f0 + static_cast<int64_t>(i) * kThreads;
     if (f >= nf4) break;
     uint32_t by, mk, na;
-    project4<FMT>(L[i], ws2, cap, by, mk, na);
+    project4<FMT>(L[i], ts, by, mk, na);
     __stcs(reinterpret_cast<unsigned int *>(pl.bytes) + f, by);
     if (pl.mask) __stcs(reinterpret_cast<unsigned int *>(pl.mask) + f, mk);
     nan_count += na;
@@ -368,17 +476,17 @@ __global__ void __launch_bounds__(kThreads) sq_merge_planes_kernel(const __grid_
                                                                       int64_t *acc) {
   __shared__ uint32_t red[kThreads / 32];
   int64_t first_block;
-  const int j = plane_of_block(t, blockIdx.x, first_block);
+  const int j = plane_of_block<kMergeF4>(t, blockIdx.x, first_block);
   const PlaneArgs &pl = t.p[j];
-  const float ws2 = pl.ws2, cap = 448.0f * pl.ws2;
+  const TensorScale ts(pl.ws2, 448.0f * pl.ws2);
   const int64_t nf4 = pl.count / 4;
-  const int64_t f0 = (static_cast<int64_t>(blockIdx.x) - first_block) * (4 * kPlaneVecs) + threadIdx.x;
+  const int64_t f0 = (static_cast<int64_t>(blockIdx.x) - first_block) * (kThreads * kMergeF4) + threadIdx.x;
   const float4 *src = reinterpret_cast<const float4 *>(pl.latent);
   uint32_t *art = reinterpret_cast<uint32_t *>(pl.bytes);
-  float4 L[kPlaneF4];
-  uint32_t old[kPlaneF4];
+  float4 L[kMergeF4];
+  uint32_t old[kMergeF4];
 #pragma unroll
-  for (int i = 0; i < kPlaneF4; ++i) {
+  for (int i = 0; i < kMergeF4; ++i) {
     const int64_t f = f0 + static_cast<int64_t>(i) * kThreads;
     if (f < nf4) {
       L[i] = __ldcs(src + f);
@@ -387,19 +495,19 @@ __global__ void __launch_bounds__(kThreads) sq_merge_planes_kernel(const __grid_
   }
   uint32_t n_changed = 0;
 #pragma unroll
-  for (int i = 0; i < kPlaneF4; ++i) {
+  for (int i = 0; i < kMergeF4; ++i) {
     const int64_t f = f0 + static_cast<int64_t>(i) * kThreads;
     if (f >= nf4) break;
     uint32_t by, mk, na;
-    project4<FMT>(L[i], ws2, cap, by, mk, na);
+    project4<FMT>(L[i], ts, by, mk, na);
     art[f] = by;
     n_changed += static_cast<uint32_t>(__popc(__vcmpne4(by, old[i]))) >> 3;  // 0xFF per differing byte
     if (pl.delta) {
-      float d[4];
-#pragma unroll
-      for (int c = 0; c < 4; ++c)
-        d[c] = __fsub_rn(scale_value<FMT>((by >> (8 * c)) & 0xFFu, ws2), scale_value<FMT>((old[i] >> (8 * c)) & 0xFFu, ws2));
-      __stcs(reinterpret_cast<float4 *>(pl.delta) + f, make_float4(d[0], d[1], d[2], d[3]));
+      float now[4], was[4];
+      scale_value4<FMT>(by, ts.b, now);
+      scale_value4<FMT>(old[i], ts.b, was);
+      __stcs(reinterpret_cast<float4 *>(pl.delta) + f, make_float4(__fsub_rn(now[0], was[0]), __fsub_rn(now[1], was[1]),
+                                                                   __fsub_rn(now[2], was[2]), __fsub_rn(now[3], was[3])));
     }
   }
   plane_counters<true>(t, j, n_changed, acc, red);
@@ -515,10 +623,10 @@ __global__ void __launch_bounds__(kThreads) sq_swap_or_diff_kernel(int64_t count
 // grouped-expert kernel") run in the same launches: expert e's planes and factors
 // follow expert e - 1's, and grid z (with the contraction chunk for the products)
 // selects the expert; a dense call is the case E = 1.
-// The three adapter kernels are register-tiled fp32 CUDA-core products: a CTA of 256
-// threads owns a 64 x 64 output tile, its operands staged in shared memory as fp32
-// (contraction index outermost), and each thread accumulates a 4 x 4 sub-tile (rows
-// ty*4 .. +3, columns tx*4 .. +3), so two 16-byte shared-memory loads feed 16 fused
+// The adapter projection of small ranks and the products for ranks above 128 and of the
+// control are register-tiled fp32 CUDA-core products: a CTA of 256 threads owns a 64 x 64 output tile, its operands staged in shared
+// memory as fp32 (contraction index outermost), and each thread accumulates a 4 x 4 sub-tile
+// (rows ty*4 .. +3, columns tx*4 .. +3), so two 16-byte shared-memory loads feed 16 fused
 // multiply-adds. Every output is summed sequentially over the contraction index, so
 // results do not change between runs.
 constexpr int kT = 64;   // output tile edge
@@ -584,6 +692,7 @@ __global__ void __launch_bounds__(kThreads) sq_project_lowrank_kernel(
 #pragma unroll
       for (int c = 0; c < 4; ++c) acc[q][c] = fmaf(bv[q], av[c], acc[q][c]);
   }
+  const TensorScale ts(ws2, cap);
   uint32_t nan_count = 0;
   // four consecutive blocks of a row per thread: one 4-byte load of the base bytes and
   // one 4-byte (16-byte for the latent) store per output where the row allows it
@@ -595,11 +704,12 @@ __global__ void __launch_bounds__(kThreads) sq_project_lowrank_kernel(
     const int64_t i0 = n * G + bq;
     if (vec && bq + 3 < G) {
       const uint32_t base4 = __ldg(reinterpret_cast<const uint32_t *>(base + i0));
-      float Lv[4];
+      float Lv[4], s[4];
+      scale_value4<FMT>(base4, ws2, s);
 #pragma unroll
-      for (int c = 0; c < 4; ++c) Lv[c] = fmaf(aor, acc[q][c], scale_value<FMT>((base4 >> (8 * c)) & 0xFFu, ws2));
+      for (int c = 0; c < 4; ++c) Lv[c] = fmaf(aor, acc[q][c], s[c]);
       uint32_t by4, mk4, na;
-      project4<FMT>(make_float4(Lv[0], Lv[1], Lv[2], Lv[3]), ws2, cap, by4, mk4, na);
+      project4<FMT>(make_float4(Lv[0], Lv[1], Lv[2], Lv[3]), ts, by4, mk4, na);
       nan_count += na;
       *reinterpret_cast<uint32_t *>(bytes_out + i0) = by4;
       if (mask_out) *reinterpret_cast<uint32_t *>(mask_out + i0) = mk4;
@@ -619,6 +729,182 @@ __global__ void __launch_bounds__(kThreads) sq_project_lowrank_kernel(
         if (latent_out) latent_out[i] = L;
         nan_count += na;
       }
+    }
+  }
+  if (nonfinite) warp_add_i32(nonfinite, nan_count);
+}
+
+// The same product and projection in larger register tiles: a CTA of 128 threads owns 64
+// rows x 128 blocks, a thread 8 rows (8 apart) x 4 consecutive blocks of each 64-wide half.
+// A shared load costs four cycles of the SM's load pipe per 16 bytes a lane reads, however
+// many lanes share an address, so the 4 x 4 tiles above are bound by their two 16-byte loads
+// per 16 multiply-adds; here four feed 64, taken two blocks at a time by packed
+// multiply-adds (the same rate as single ones, in half the issue slots). B and A are staged
+// as fp32 as they lie: a 16-byte load of B holds four j of a row, one of A four blocks of a
+// j. Ranks above kWideChunk run chunk by chunk on the same accumulators.
+// Measured, against the 4 x 4 tiles: 14336 x 256 blocks at rank 58 20.7 against 26.7 us, 128
+// experts of 768 x 128 at rank 54 65 against 84 us; but 4096 x 256 at rank 16 11.0 against
+// 8.8 us, 1024 x 256 at rank 128 (32 tiles) 22 against 16 us and 128 experts of 2048 x 48 at
+// rank 54 126 against 103 us, so small ranks and grids and narrow planes stay there, and with
+// them planes whose rows are not whole groups of four blocks.
+constexpr int kWideThreads = 128, kWideRows = 64, kWideCols = 128;
+constexpr int kWideChunk = 64;  // j per chunk
+// Bytes of a staged B row: the 16-byte units are odd in number, so that the four rows a
+// warp reads at a time lie in different banks.
+__host__ __device__ constexpr int wide_pitch(int len) { return (((len + 3) / 4) | 1) * 16; }
+__host__ __device__ constexpr int wide_smem(int r) {
+  const int len = r < kWideChunk ? r : kWideChunk;
+  return kWideRows * wide_pitch(len) + len * kWideCols * 4;
+}
+
+template <int FMT>
+__global__ void __launch_bounds__(kWideThreads, 3) sq_project_lowrank_wide_kernel(
+    int64_t N, int64_t G, int r, float ws2, float cap, const float *__restrict__ ws2_per, float aor,
+    const uint8_t *__restrict__ base, const uint16_t *__restrict__ B, const uint16_t *__restrict__ A,
+    uint8_t *__restrict__ bytes_out, uint8_t *__restrict__ mask_out, int32_t *__restrict__ nonfinite,
+    float *__restrict__ latent_out) {
+  constexpr int CG = 2, kCols = kWideCols;
+  extern __shared__ __align__(16) uint8_t lr_bytes[];
+  const int64_t n0 = static_cast<int64_t>(blockIdx.x) * kWideRows;
+  const int64_t b0 = static_cast<int64_t>(blockIdx.y) * kCols;
+  // expert blockIdx.z: its planes, factors and (NVFP4 experts) tensor scale
+  const int64_t e = blockIdx.z, plane = N * G;
+  base += e * plane;
+  B += e * N * r;
+  A += e * r * G;
+  bytes_out += e * plane;
+  if (mask_out) mask_out += e * plane;
+  if (latent_out) latent_out += e * plane;
+  if (ws2_per) {
+    ws2 = __ldg(ws2_per + e);
+    cap = 448.0f * ws2;  // the same IEEE fp32 product as the host's single-plane cap
+  }
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int ty = (warp >> 1) * 4 + (lane >> 3), tx = (warp & 1) * 8 + (lane & 7);
+  const int pitch = wide_pitch(r < kWideChunk ? r : kWideChunk);
+  float *sA = reinterpret_cast<float *>(lr_bytes + kWideRows * pitch);  // [j][kCols]
+  uint64_t acc[8][2 * CG];
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+#pragma unroll
+    for (int c = 0; c < 2 * CG; ++c) acc[i][c] = 0;
+  for (int j0 = 0; j0 < r; j0 += kWideChunk) {
+    const int len = r - j0 < kWideChunk ? r - j0 : kWideChunk;
+    if (j0 > 0) __syncthreads();  // the previous chunk is used up
+    // Staging: the loads of a chunk are issued before its stores. B: pairs (j, j + 1) of row
+    // `row`; (row, pair) of the thread's k-th pair advance without dividing.
+    const int pairs = (len + 1) / 2;
+    const int drow = kWideThreads / pairs, dq = kWideThreads % pairs;
+    const int row0 = static_cast<int>(threadIdx.x) / pairs, q0 = static_cast<int>(threadIdx.x) % pairs;
+    constexpr int kB = kWideRows * (kWideChunk / 2) / kWideThreads, kA = 8 * CG;
+    uint32_t wb[kB];
+    const bool even = (r & 1) == 0;  // pairs are 4-byte aligned
+#pragma unroll
+    for (int k = 0, row = row0, q = q0; k < kB; ++k) {
+      wb[k] = 0;
+      if (row < kWideRows && n0 + row < N) {
+        const uint16_t *src = B + (n0 + row) * r + j0 + 2 * q;
+        if (even) {
+          wb[k] = __ldg(reinterpret_cast<const uint32_t *>(src));
+        } else {
+          wb[k] = __ldg(src);
+          if (2 * q + 1 < len) wb[k] |= static_cast<uint32_t>(__ldg(src + 1)) << 16;
+        }
+      }
+      row += drow;
+      q += dq;
+      if (q >= pairs) {
+        q -= pairs;
+        ++row;
+      }
+    }
+    {  // A: four blocks of a j at a time
+      uint2 wa[kA];
+#pragma unroll
+      for (int k = 0; k < kA; ++k) {
+        const int i = threadIdx.x + kWideThreads * k;
+        const int j = i / (kCols / 4), c = 4 * (i % (kCols / 4));
+        wa[k] = make_uint2(0, 0);
+        if (j >= len) continue;
+        const uint16_t *src = A + static_cast<int64_t>(j0 + j) * G + b0 + c;
+        if (b0 + c < G) wa[k] = __ldg(reinterpret_cast<const uint2 *>(src));  // G is a multiple of 4
+      }
+#pragma unroll
+      for (int k = 0; k < kA; ++k) {
+        const int i = threadIdx.x + kWideThreads * k;
+        const int j = i / (kCols / 4), c = 4 * (i % (kCols / 4));
+        if (j < len)
+          *reinterpret_cast<float4 *>(sA + j * kCols + c) =
+              make_float4(__uint_as_float(wa[k].x << 16), __uint_as_float(wa[k].x & 0xFFFF0000u),
+                          __uint_as_float(wa[k].y << 16), __uint_as_float(wa[k].y & 0xFFFF0000u));
+      }
+    }
+#pragma unroll
+    for (int k = 0, row = row0, q = q0; k < kB; ++k) {
+      if (row < kWideRows)
+        *reinterpret_cast<uint2 *>(lr_bytes + row * pitch + 8 * q) = make_uint2(wb[k] << 16, wb[k] & 0xFFFF0000u);
+      row += drow;
+      q += dq;
+      if (q >= pairs) {
+        q -= pairs;
+        ++row;
+      }
+    }
+    __syncthreads();
+    const uint8_t *pb = lr_bytes + ty * pitch;
+    const float *pa = sA + tx * 4;
+#pragma unroll 1
+    for (int j = 0; j < len; j += 4) {
+      float4 b[8];  // past an odd length: staged or stale values that no multiply-add takes
+#pragma unroll
+      for (int i = 0; i < 8; ++i) b[i] = *reinterpret_cast<const float4 *>(pb + i * 8 * pitch + 4 * j);
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        if (t > 0 && j + t >= len) break;
+        ulonglong2 a[CG];
+#pragma unroll
+        for (int c = 0; c < CG; ++c) a[c] = *reinterpret_cast<const ulonglong2 *>(pa + (j + t) * kCols + 64 * c);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const float bt = t == 0 ? b[i].x : t == 1 ? b[i].y : t == 2 ? b[i].z : b[i].w;
+          const uint64_t bb = dup_x2(bt);
+#pragma unroll
+          for (int c = 0; c < CG; ++c) {
+            acc[i][2 * c] = fma_x2(bb, a[c].x, acc[i][2 * c]);
+            acc[i][2 * c + 1] = fma_x2(bb, a[c].y, acc[i][2 * c + 1]);
+          }
+        }
+      }
+    }
+  }
+  const TensorScale ts(ws2, cap);
+  const uint64_t aor2 = dup_x2(aor);
+  uint32_t nan_count = 0;
+  const int rows_left = static_cast<int>(N - n0 - ty < kWideRows ? N - n0 - ty : kWideRows);
+#pragma unroll
+  for (int g = 0; g < CG; ++g) {
+    const int64_t bq = b0 + 64 * g + tx * 4;
+    if (bq >= G) break;
+    const int64_t first = (n0 + ty) * G + bq;
+    uint32_t old[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      if (8 * i < rows_left) old[i] = __ldg(reinterpret_cast<const uint32_t *>(base + first + 8 * i * G));
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      if (8 * i >= rows_left) break;
+      const int64_t i0 = first + 8 * i * G;
+      float s[4];
+      scale_value4<FMT>(old[i], ws2, s);
+      const uint64_t l01 = fma_x2(aor2, acc[i][2 * g], pair_x2(s[0], s[1]));
+      const uint64_t l23 = fma_x2(aor2, acc[i][2 * g + 1], pair_x2(s[2], s[3]));
+      const float4 L = make_float4(lo_x2(l01), hi_x2(l01), lo_x2(l23), hi_x2(l23));
+      uint32_t by4, mk4, na;
+      project4<FMT>(L, ts, by4, mk4, na);
+      nan_count += na;
+      *reinterpret_cast<uint32_t *>(bytes_out + i0) = by4;
+      if (mask_out) *reinterpret_cast<uint32_t *>(mask_out + i0) = mk4;
+      if (latent_out) *reinterpret_cast<float4 *>(latent_out + i0) = L;
     }
   }
   if (nonfinite) warp_add_i32(nonfinite, nan_count);
@@ -988,14 +1274,14 @@ cudaError_t launch_merge(int fmt, int64_t count, float ws2, const float *latent,
   return cudaGetLastError();
 }
 
-static unsigned planes_grid(const PlaneTable &t) {
+static unsigned planes_grid(const PlaneTable &t, int f4) {
   int64_t g = 0;
-  for (int j = 0; j < t.n; ++j) g += (t.p[j].count / 16 + kPlaneVecs - 1) / kPlaneVecs;
+  for (int j = 0; j < t.n; ++j) g += plane_ctas(t.p[j].count, f4);
   return static_cast<unsigned>(g);
 }
 
 cudaError_t launch_project_planes(int fmt, const PlaneTable &t, int64_t *acc, cudaStream_t stream) {
-  const unsigned grid = planes_grid(t);
+  const unsigned grid = planes_grid(t, kProjectF4);
   if (grid == 0) {  // no blocks at all: the counters still receive 0
     for (int j = 0; j < t.n; ++j)
       if (t.p[j].counter) {
@@ -1012,7 +1298,7 @@ cudaError_t launch_project_planes(int fmt, const PlaneTable &t, int64_t *acc, cu
 }
 
 cudaError_t launch_merge_planes(int fmt, const PlaneTable &t, int64_t *acc, cudaStream_t stream) {
-  const unsigned grid = planes_grid(t);
+  const unsigned grid = planes_grid(t, kMergeF4);
   if (grid == 0) {
     for (int j = 0; j < t.n; ++j)
       if (t.p[j].counter) {
@@ -1028,15 +1314,41 @@ cudaError_t launch_merge_planes(int fmt, const PlaneTable &t, int64_t *acc, cuda
   return cudaGetLastError();
 }
 
+template <int FMT>
+static cudaError_t launch_wide(int64_t N, int64_t G, int r, float ws2, float cap, const float *ws2_per,
+                               float alpha_over_r, const uint8_t *base, const uint16_t *B, const uint16_t *A,
+                               uint8_t *bytes_out, uint8_t *mask_out, int32_t *nonfinite, float *latent_out,
+                               cudaStream_t stream, int experts) {
+  const dim3 grid(static_cast<unsigned>((N + kWideRows - 1) / kWideRows),
+                  static_cast<unsigned>((G + kWideCols - 1) / kWideCols), static_cast<unsigned>(experts));
+  const int smem = wide_smem(r);  // <= 50 KiB
+  const cudaError_t e = cudaFuncSetAttribute(sq_project_lowrank_wide_kernel<FMT>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  sq_project_lowrank_wide_kernel<FMT><<<grid, kWideThreads, smem, stream>>>(N, G, r, ws2, cap, ws2_per, alpha_over_r,
+                                                                            base, B, A, bytes_out, mask_out, nonfinite,
+                                                                            latent_out);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_project_lowrank(int fmt, int64_t N, int64_t G, int r, float ws2, float alpha_over_r,
                                    const uint8_t *base, const uint16_t *B, const uint16_t *A, uint8_t *bytes_out,
-                                   uint8_t *mask_out, int32_t *nonfinite, float *latent_out, cudaStream_t stream,
-                                   int experts, const float *ws2_per) {
+                                   uint8_t *mask_out, int32_t *nonfinite, float *latent_out, int sm_count,
+                                   cudaStream_t stream, int experts, const float *ws2_per) {
   if (nonfinite) {
     cudaError_t e = cudaMemsetAsync(nonfinite, 0, sizeof(int32_t), stream);
     if (e != cudaSuccess) return e;
   }
   const float cap = 448.0f * ws2;  // one IEEE fp32 multiply
+  // the larger tiles where the products outweigh the projection, there are two tiles per SM
+  // and three quarters of the tiles' columns are blocks
+  const int64_t wide_cols = (G + kWideCols - 1) / kWideCols;
+  const int64_t wide_ctas = (N + kWideRows - 1) / kWideRows * wide_cols * experts;
+  if (r >= 32 && G % 4 == 0 && wide_ctas >= 2 * sm_count && 3 * wide_cols * kWideCols <= 4 * G)
+    return fmt == 0 ? launch_wide<0>(N, G, r, ws2, cap, ws2_per, alpha_over_r, base, B, A, bytes_out, mask_out,
+                                     nonfinite, latent_out, stream, experts)
+                    : launch_wide<1>(N, G, r, ws2, cap, nullptr, alpha_over_r, base, B, A, bytes_out, mask_out,
+                                     nonfinite, latent_out, stream, experts);
   const dim3 grid(static_cast<unsigned>((N + kT - 1) / kT), static_cast<unsigned>((G + kT - 1) / kT),
                   static_cast<unsigned>(experts));
   const size_t smem = static_cast<size_t>(kTP + kT) * r * sizeof(float);  // <= 132 KiB for r <= 256
