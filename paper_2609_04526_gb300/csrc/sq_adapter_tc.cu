@@ -16,6 +16,11 @@
 // CTA covers all blocks, else per part and added in part order; the partial dA of a
 // row chunk is added over the chunks in chunk order. Fixed order throughout, so
 // reruns give identical bits.
+//
+// Bound by each CTA's chain of staging, MMAs and drain (two CTAs per SM), so its length in
+// instructions counts: B's staging without divisions, two values split per conversion and
+// the 36 MMAs of a step issued from uniform registers took the kernel from 50 to 41 us for
+// the 128 experts of 768 x 128 blocks at rank 54 (75 MB in and out: 11 us of memory time).
 #include "sq_gemm_kernels.cuh"
 
 namespace sqi {
@@ -46,17 +51,23 @@ __device__ __forceinline__ void sts32(uint32_t addr, uint32_t v) {
   asm volatile("st.shared.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
 
-__device__ __forceinline__ uint32_t bf16_rn(float x) {
-  return static_cast<uint32_t>(__bfloat16_as_ushort(__float2bfloat16_rn(x)));
+// Two fp32 -> a pair of bf16, round to nearest even, `lo` in the low half.
+__device__ __forceinline__ uint32_t bf16x2_rn(float lo, float hi) {
+  uint32_t d;
+  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(hi), "f"(lo));
+  return d;
 }
 
-// x = hi + mid + lo, each a bf16 (round to nearest even), the remainders exact in fp32.
-__device__ __forceinline__ void split3(float x, uint32_t &hi, uint32_t &mid, uint32_t &lo) {
-  hi = bf16_rn(x);
-  const float r1 = __fsub_rn(x, __uint_as_float(hi << 16));
-  mid = bf16_rn(r1);
-  const float r2 = __fsub_rn(r1, __uint_as_float(mid << 16));
-  lo = bf16_rn(r2);
+// x = hi + mid + lo for two neighbours, each part a bf16 (round to nearest even), the
+// remainders exact in fp32.
+__device__ __forceinline__ void split3(float x0, float x1, uint32_t &hi, uint32_t &mid, uint32_t &lo) {
+  hi = bf16x2_rn(x0, x1);
+  x0 = __fsub_rn(x0, __uint_as_float(hi << 16));
+  x1 = __fsub_rn(x1, __uint_as_float(hi & 0xFFFF0000u));
+  mid = bf16x2_rn(x0, x1);
+  x0 = __fsub_rn(x0, __uint_as_float(mid << 16));
+  x1 = __fsub_rn(x1, __uint_as_float(mid & 0xFFFF0000u));
+  lo = bf16x2_rn(x0, x1);
 }
 
 // grid (ceil(N / 128), parts * experts): CTA (c, p, e) covers rows 128 c .. + 127 and
@@ -129,6 +140,7 @@ __global__ void __launch_bounds__(kAtThreads, 2)
     // 32 in flight per thread before the stores; rows past N and j >= r stay zero below
     const int pairs = r / 2, words = kAtRows * pairs;
     const int64_t rows_here = N - n0 < kAtRows ? N - n0 : kAtRows;
+    const int here = static_cast<int>(rows_here) * pairs;  // words of the rows that exist
     const uint32_t *src = reinterpret_cast<const uint32_t *>(Bm + n0 * r);  // 4-byte aligned: r even
     // zero fill of the pairs' 16-byte chunks that hold no data (j >= r rounded to 8, rows past N)
     for (int u = threadIdx.x; u < kAtRows * 16; u += kAtThreads) {
@@ -143,20 +155,27 @@ __global__ void __launch_bounds__(kAtThreads, 2)
       }
     }
     __syncthreads();  // zeros before the data words that share their chunks
+    // (row, pair) of a thread's words advance by (kAtThreads / pairs, kAtThreads % pairs)
+    const int drow = kAtThreads / pairs, dq = kAtThreads % pairs;
+    int nn = static_cast<int>(threadIdx.x) / pairs, jp = static_cast<int>(threadIdx.x) % pairs;
     for (int w0 = 0; w0 < words; w0 += 16 * kAtThreads) {
       uint32_t v[16];
 #pragma unroll
       for (int q = 0; q < 16; ++q) {
         const int w = w0 + q * kAtThreads + threadIdx.x;
-        v[q] = (w < words && w / pairs < rows_here) ? __ldg(src + w) : 0u;
+        v[q] = w < here ? __ldg(src + w) : 0u;
       }
 #pragma unroll
       for (int q = 0; q < 16; ++q) {
-        const int w = w0 + q * kAtThreads + threadIdx.x;
-        if (w < words && w / pairs < rows_here) {
-          const int nn = w / pairs, j = 2 * (w - nn * pairs);
-          const int ch = j >> 3;
-          sts32(base + S::kOffB + (ch >> 3) * S::kTile + sw128_chunk(nn, ch & 7) + (j & 7) * 2, v[q]);
+        if (w0 + q * kAtThreads + static_cast<int>(threadIdx.x) < here) {
+          const int ch = jp >> 2;
+          sts32(base + S::kOffB + (ch >> 3) * S::kTile + sw128_chunk(nn, ch & 7) + (jp & 3) * 4, v[q]);
+        }
+        nn += drow;
+        jp += dq;
+        if (jp >= pairs) {
+          jp -= pairs;
+          ++nn;
         }
       }
     }
@@ -207,14 +226,7 @@ __global__ void __launch_bounds__(kAtThreads, 2)
       const int nn = (threadIdx.x >> 3) + (kAtThreads / 8) * i;
       uint32_t hi[4], mid[4], lo[4];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        uint32_t h0, m0, l0, h1, m1, l1;
-        split3(gv[i][2 * q], h0, m0, l0);
-        split3(gv[i][2 * q + 1], h1, m1, l1);
-        hi[q] = h0 | (h1 << 16);
-        mid[q] = m0 | (m1 << 16);
-        lo[q] = l0 | (l1 << 16);
-      }
+      for (int q = 0; q < 4; ++q) split3(gv[i][2 * q], gv[i][2 * q + 1], hi[q], mid[q], lo[q]);
       const uint32_t off = sw128_chunk(nn, threadIdx.x & 7);
       st_shared_v4(base + S::kOffG + off, hi[0], hi[1], hi[2], hi[3]);
       st_shared_v4(base + S::kOffG + S::kTile + off, mid[0], mid[1], mid[2], mid[3]);
@@ -253,7 +265,7 @@ __global__ void __launch_bounds__(kAtThreads, 2)
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (warp == 0) {
       tc_fence_after();
       // dB[n, j] += sum_b part[n, b] A[j, b]: 4 K-steps of 16 blocks, three parts each
 #pragma unroll
@@ -261,7 +273,7 @@ __global__ void __launch_bounds__(kAtThreads, 2)
         const uint64_t bdesc = smem_desc_sw128(base + S::kOffA + kk * 32, 16, 1024);
 #pragma unroll
         for (int pt = 0; pt < 3; ++pt)
-          umma_bf16(tmem, smem_desc_sw128(base + S::kOffG + pt * S::kTile + kk * 32, 16, 1024), bdesc, idesc_db,
+          umma_bf16_elect(tmem, smem_desc_sw128(base + S::kOffG + pt * S::kTile + kk * 32, 16, 1024), bdesc, idesc_db,
                     (s > 0 || kk > 0 || pt > 0) ? 1u : 0u);
       }
       // dA step [j, b] = sum_n B[n, j] part[n, b]: 8 K-steps of 16 rows n (2 KiB), three parts
@@ -271,10 +283,10 @@ __global__ void __launch_bounds__(kAtThreads, 2)
         const uint64_t adesc = smem_desc_sw128(base + S::kOffB + kk * 2048, S::kTile, 1024);
 #pragma unroll
         for (int pt = 0; pt < 3; ++pt)
-          umma_bf16(d_da, adesc, smem_desc_sw128(base + S::kOffG + pt * S::kTile + kk * 2048, S::kTile, 1024),
+          umma_bf16_elect(d_da, adesc, smem_desc_sw128(base + S::kOffG + pt * S::kTile + kk * 2048, S::kTile, 1024),
                     idesc_da, (kk > 0 || pt > 0) ? 1u : 0u);
       }
-      umma_commit(bar);
+      umma_commit_elect(bar);
     }
     if (s + 1 < steps) load(s + 1);  // in flight during the MMAs
     if (!(ok = mbar_wait(bar, static_cast<uint32_t>(s) & 1u, abort_flag, err))) break;

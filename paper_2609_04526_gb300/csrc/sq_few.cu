@@ -61,25 +61,7 @@ struct FewMaps {
   CUtensorMap codes;   // the packed codes in 64-byte x 128-row boxes
 };
 
-// MMAs, commits, barrier arrivals and TMA loads issued by one elected lane of a converged warp.
-__device__ __forceinline__ void umma_bf16_elect(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                                uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p, e;\n\t"
-      "elect.sync _|e, 0xFFFFFFFF;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-__device__ __forceinline__ void umma_commit_elect(uint64_t *bar) {
-  asm volatile(
-      "{\n\t.reg .pred e;\n\t"
-      "elect.sync _|e, 0xFFFFFFFF;\n\t"
-      "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(smem_u32(bar))
-      : "memory");
-}
-
+// Barrier arrivals and TMA loads issued by one elected lane of a converged warp.
 __device__ __forceinline__ void expect_tx_elect(uint64_t *bar, uint32_t bytes) {
   asm volatile(
       "{\n\t.reg .pred e;\n\t"
