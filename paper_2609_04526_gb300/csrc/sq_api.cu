@@ -301,7 +301,7 @@ sq_status run_gemm(sq_handle h, int mode, const sq_weight *w, const void *a_ptr,
       return run_few(h, dev, mode, w->fmt, 1, w->N, w->K, w->codes, w->scales, w->ws2, a_ptr, M, out, nullptr,
                      tiles_at(limit), sqi::few_tile_tokens(M, limit), stream);
   }
-  CUtensorMap tmA, tmB, tmOut;
+  CUtensorMap tmA, tmB, tmC;
   const int64_t K2 = w->K / 2;  // code bytes per row
   if (mode == sqi::MODE_FWD) {
     SQ_TRY(make_act_map(h, &tmA, a_ptr, w->K, M, 64, sqi::kBM));  // X, 128 x 64 K-major boxes
@@ -309,18 +309,20 @@ sq_status run_gemm(sq_handle h, int mode, const sq_weight *w, const void *a_ptr,
     SQ_TRY(make_map(h, &tmB, w->codes, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, K2, w->N, 64, 128,
                     CU_TENSOR_MAP_SWIZZLE_64B));
     // Y [M, N]: 32-row x 32-column store boxes (the epilogue's staging tiles), 64-byte swizzle
-    SQ_TRY(make_out_map(h, &tmOut, out, w->N, M));
+    SQ_TRY(make_out_map(h, &tmC, out, w->N, M));
   } else if (mode == sqi::MODE_DX) {
     SQ_TRY(make_act_map(h, &tmA, a_ptr, w->N, M, 64, sqi::kBM));  // dY, 128 x 64 K-major boxes
     // codes: 128 contraction rows x 64 bytes (128 weights) per stage and CTA, 64-byte swizzle
     SQ_TRY(make_map(h, &tmB, w->codes, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, K2, w->N, 64, 128,
                     CU_TENSOR_MAP_SWIZZLE_64B));
     // dX [M, K]: the same store boxes
-    SQ_TRY(make_out_map(h, &tmOut, out, w->K, M));
+    SQ_TRY(make_out_map(h, &tmC, out, w->K, M));
   } else {
     // dY and X as MN-major boxes of 64 features x kSgradBK tokens
     SQ_TRY(make_act_map(h, &tmA, a_ptr, w->N, M, 64, sqi::kSgradBK));
     SQ_TRY(make_act_map(h, &tmB, b_ptr, w->K, M, 64, sqi::kSgradBK));
+    SQ_TRY(make_map(h, &tmC, w->codes, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, K2, w->N, 64, 128,
+                    CU_TENSOR_MAP_SWIZZLE_64B));
   }
   sqi::GemmArgs a;
   a.mode = mode;
@@ -343,7 +345,7 @@ sq_status run_gemm(sq_handle h, int mode, const sq_weight *w, const void *a_ptr,
       a.partial = static_cast<float *>(dev->partial.ptr);
     }
   }
-  cudaError_t e = sqi::launch_gemm(a, tmA, tmB, mode == sqi::MODE_SGRAD ? nullptr : &tmOut, dev->sm_count, stream);
+  cudaError_t e = sqi::launch_gemm(a, tmA, tmB, tmC, dev->sm_count, stream);
   if (e != cudaSuccess) return cuda_fail(h, e, "kernel launch");
   return SQ_OK;
 }

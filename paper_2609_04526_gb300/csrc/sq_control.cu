@@ -22,7 +22,7 @@ cudaError_t launch_control(const GemmArgs &a, const CUtensorMap &tmA, const CUte
   p.total = p.tiles_m * p.tiles_n;
   if (a.mode == MODE_FWD) return launch_pair<MODE_FWD, kFmtBf16Mul, false>(p, tmA, tmB, *tmOut, sm_count, stream);
   if (a.mode == MODE_DX) return launch_pair<MODE_DX, kFmtBf16Mul, false>(p, tmA, tmB, *tmOut, sm_count, stream);
-  return launch_sgrad<kFmtBf16Mul, false>(p, tmA, tmB, sm_count, stream);
+  return launch_sgrad<kFmtBf16Mul, false>(p, tmA, tmB, tmA, sm_count, stream);
 }
 
 }  // namespace sqi

@@ -30,9 +30,8 @@ __global__ void sq_split_reduce_kernel(const float *__restrict__ partial, int sp
   }
 }
 
-cudaError_t launch_gemm(const GemmArgs &a, const CUtensorMap &tmA, const CUtensorMap &tmB, const CUtensorMap *tmOut,
+cudaError_t launch_gemm(const GemmArgs &a, const CUtensorMap &tmA, const CUtensorMap &tmB, const CUtensorMap &tmC,
                         int sm_count, cudaStream_t stream) {
-  if (a.mode != MODE_SGRAD && !tmOut) return cudaErrorInvalidValue;
   KParams p{a.codes, a.scales, a.ws2, a.M, a.N, a.K, a.out, a.mask, a.err, 0, 0, 0, nullptr, 1};
   if (a.mode == MODE_SGRAD) {
     p.tiles_m = static_cast<int>((a.N + kSgradTile - 1) / kSgradTile);
@@ -44,10 +43,10 @@ cudaError_t launch_gemm(const GemmArgs &a, const CUtensorMap &tmA, const CUtenso
   }
   p.total = p.tiles_m * p.tiles_n;
   if (a.mode != MODE_SGRAD) {
-    if (a.fmt == 0 && a.mode == MODE_FWD) return launch_pair<MODE_FWD, 0, false>(p, tmA, tmB, *tmOut, sm_count, stream);
-    if (a.fmt == 0) return launch_pair<MODE_DX, 0, false>(p, tmA, tmB, *tmOut, sm_count, stream);
-    if (a.mode == MODE_FWD) return launch_pair<MODE_FWD, 1, false>(p, tmA, tmB, *tmOut, sm_count, stream);
-    return launch_pair<MODE_DX, 1, false>(p, tmA, tmB, *tmOut, sm_count, stream);
+    if (a.fmt == 0 && a.mode == MODE_FWD) return launch_pair<MODE_FWD, 0, false>(p, tmA, tmB, tmC, sm_count, stream);
+    if (a.fmt == 0) return launch_pair<MODE_DX, 0, false>(p, tmA, tmB, tmC, sm_count, stream);
+    if (a.mode == MODE_FWD) return launch_pair<MODE_FWD, 1, false>(p, tmA, tmB, tmC, sm_count, stream);
+    return launch_pair<MODE_DX, 1, false>(p, tmA, tmB, tmC, sm_count, stream);
   }
   if (a.splits > 1) {
     if (!a.partial || a.splits > kMaxSgradSplits) return cudaErrorInvalidValue;
@@ -55,8 +54,8 @@ cudaError_t launch_gemm(const GemmArgs &a, const CUtensorMap &tmA, const CUtenso
     p.partial = a.partial;
     p.total *= a.splits;
   }
-  cudaError_t e = a.fmt == 0 ? launch_sgrad<0, false>(p, tmA, tmB, sm_count, stream)
-                             : launch_sgrad<1, false>(p, tmA, tmB, sm_count, stream);
+  cudaError_t e = a.fmt == 0 ? launch_sgrad<0, false>(p, tmA, tmB, tmC, sm_count, stream)
+                             : launch_sgrad<1, false>(p, tmA, tmB, tmC, sm_count, stream);
   if (e != cudaSuccess || a.splits <= 1) return e;
   const int64_t count = a.N * (a.K / (a.fmt == 0 ? 16 : 32));
   const int64_t blocks = (count / 4 + 255) / 256;

@@ -1367,20 +1367,30 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg::kThreads, 1
 // its TMEM and reduces it by blocks in its own epilogue.
 //
 // A unit of few tokens (an expert's rows, a short example) is bound by the epilogue:
-// eight warps share it (two per TMEM lane quadrant, one per column half), each lane
-// fetches its codes and mask bytes of the NEXT unit before it works on this one, the
-// TMEM load of a column group runs under the previous group's arithmetic, and the
-// accumulator is released once its last group is in registers. With four warps that
-// loaded a group's codes only after its accumulator, a 256-token unit took ~8,600
-// cycles for 2,048 cycles of MMAs; the scale gradient of 128 experts of 2880 x 2880
-// with 256 rows each went from 1100 to 630 us, of 128 experts of 768 x 2048 with 128
-// rows each from 196 to 142 us, and of a 4096 x 4096 linear with 187 tokens from 23.7
-// to 17.8 us; long contractions (2,000 tokens and more a unit) are unchanged.
+//  - sixteen warps share it (four per TMEM lane quadrant, 64 columns each);
+//  - the codes come by TMA, and each lane's mask bytes as one word, a unit ahead. A row of
+//    the tile lies in lines of its own, so a load by 32 lanes is 32 requests to the L1
+//    however wide it is, and sixteen warps that fetched codes and mask bytes themselves
+//    spent 3,000 of a unit's 7,000 cycles there;
+//  - a unit's place comes from steps and tables in shared memory instead of divisions;
+//  - the TMEM load of a column group runs under the previous group's arithmetic, and the
+//    accumulator is released once its last group is in registers.
+// With four warps that loaded a group's codes only after its accumulator, a 256-token unit
+// took ~8,600 cycles for 2,048 cycles of MMAs; with eight that fetched a unit ahead, ~5,000.
+// Scale gradients, four warps / eight / now: 128 experts of 2880 x 2880 with 256 rows each
+// 1106 / 620 / 540 us, of 768 x 2048 with 128 rows each 207 / 125 / 89 us, with 32 rows
+// each 205 / 125 / 85 us, a 4096 x 4096 linear with 187 tokens 22.5 / 17 / 14.5 us, a
+// 14336 x 4096 one with 300 tokens 55 / 39 / 35 us; long contractions (2,000 tokens and more
+// a unit) are unchanged at the MMAs' rate. Measured and not kept: units dealt to two sets of
+// eight warps (616 us in the first case), stages of 64 or 96 tokens (630, 585), codes on
+// their way to L2 a unit before (no change), mask bytes gathered by one warp for the sixteen
+// (122 us in the second: one slot's latency is then on the path of every unit).
 struct SgradPairCfg {
-  static constexpr int kEpiWarps = 8;  // warp w: TMEM lanes 32 (w % 4) .. + 31, columns 128 (w / 4) .. + 127
+  static constexpr int kEpiWarps = 16;  // warp w: TMEM lanes 32 (w % 4) .. + 31, columns 64 (w / 4) .. + 63
   static constexpr int kTmaWarp = kEpiWarps;
   static constexpr int kMmaWarp = kTmaWarp + 1;
-  static constexpr int kThreads = 32 * (kMmaWarp + 1);
+  static constexpr int kCodeWarp = kMmaWarp + 1;  // packed codes
+  static constexpr int kThreads = 32 * (kCodeWarp + 1);
   static constexpr int kBK = kSgradBK;         // tokens per stage: 8 MMAs of K = 16
   static constexpr int kStages = 3;
   static constexpr int kA = 128 * kBK * 2;     // 16 KiB: this CTA's 128 n-rows of dY^T, two MN atoms of 64 n
@@ -1389,26 +1399,36 @@ struct SgradPairCfg {
   static constexpr int kStageBytes = kA + kB;
   static constexpr uint32_t kTx = 2 * kStageBytes;  // both CTAs' tiles, counted on the leader's barrier
   static constexpr int kTile = kSgradTile;
-  static constexpr int kSmemBytes = kStages * kStageBytes + 1024 + 1024;
+  static constexpr int kCached = 1024;         // experts (rows, ids) and tiles of a plane kept in shared memory
+  static constexpr int kCodes = 128 * kTile / 2;                  // this CTA's codes of a unit, two 64-byte-wide boxes
+  static constexpr int kOffCodes = kStages * kStageBytes;
+  static constexpr int kOffBar = kOffCodes + kCodes;
+  static constexpr int kOffTable = kOffBar + 256;                 // ... expert and tile tables
+  static constexpr int kSmemBytes = kOffTable + kCached * 12 + 1024;
 };
+static_assert(SgradPairCfg::kTile == 256, "an epilogue warp takes 64 columns: two 16-byte code chunks of a row");
+static_assert(SgradPairCfg::kOffCodes % 1024 == 0, "swizzled code boxes");
 static_assert(SgradPairCfg::kSmemBytes <= 232448, "scale-gradient kernel exceeds the opt-in shared memory");
 
 template <int FMT, bool GR>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(SgradPairCfg::kThreads, 1)
     sq_sgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                         const KParams p) {
+                         const __grid_constant__ CUtensorMap tmC, const KParams p) {
   using C = SgradPairCfg;
   constexpr int S = C::kStages;
   constexpr int B = FMT == 1 ? 32 : 16;  // the multiplicative control has one factor per 16 weights
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint64_t *bars = reinterpret_cast<uint64_t *>(smem + S * C::kStageBytes);
+  uint8_t *s_codes = smem + C::kOffCodes;
+  uint64_t *bars = reinterpret_cast<uint64_t *>(smem + C::kOffBar);
   uint64_t *full = bars;              // [S] leader: both CTAs' tiles of the stage landed (1 arrival + tx)
   uint64_t *empty = full + S;         // [S] pair MMAs reading the stage completed     (multicast commit)
   uint64_t *tfull = empty + S;        // [2] accumulator buffer complete                (multicast commit)
   uint64_t *tempty = tfull + 2;       // [2] leader: both epilogues drained the buffer
                                       //     (kEpiWarps arrivals + the peer warps' st.async tx)
-  uint64_t *drain = tempty + 2;
+  uint64_t *cfull = tempty + 2;       // codes of the unit landed                       (1 arrival + tx)
+  uint64_t *cempty = cfull + 1;       // every epilogue warp took them into registers
+  uint64_t *drain = cempty + 1;
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(drain + 1);
   volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
   uint32_t *sink = reinterpret_cast<uint32_t *>(drain + 2);  // [kEpiWarps] leader: st.async targets
@@ -1421,25 +1441,43 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(SgradPairCfg::kThrea
   const int total = p.total;
   // Unit u of the launch: tile (tm, tn) (of expert e in a grouped launch) over the
   // token stages [m0, m0 + kBK * num_k): all M tokens, the expert's own M_e, or in
-  // a dense launch cut into token splits, part sp of them (an expert or part
-  // without tokens gets zero gradient blocks). Returns num_k; `len` are its tokens.
-  const int tiles_per_split = p.tiles_m * p.tiles_n;
+  // a dense launch cut into token splits, part e of them (an expert or part without tokens
+  // gets zero gradient blocks). Each role walks its units step by step: entry and tile index
+  // advance by the quotient and rest of the stride, and the tile's coordinates, the experts'
+  // row counts and their ids come from shared memory (the streams of codes push a global
+  // table out of the L1 that is left). With a division per unit, the epilogue's 16 warps
+  // spent a fifth of a short unit on it.
+  struct Unit {
+    int e, local;  // table entry or token part, tile of it
+  };
+  const int per = p.tiles_m * p.tiles_n;
+  auto advance = [&](Unit &w, const Unit &by) {
+    w.e += by.e;
+    w.local += by.local;
+    if (w.local >= per) {
+      w.local -= per;
+      ++w.e;
+    }
+  };
+  int *s_rows = reinterpret_cast<int *>(smem + C::kOffTable), *s_ids = s_rows + C::kCached;
+  int *s_tiles = s_ids + C::kCached;
+  const int cached = GR ? min(p.groups, C::kCached) : 0;
+  auto tile_of = [&](int local, int &tm, int &tn) {
+    if (local < C::kCached) {
+      tm = s_tiles[local] & 0xFFFF;
+      tn = s_tiles[local] >> 16;
+    } else {
+      tile_coords<kSgradGroup>(local, p.tiles_m, p.tiles_n, tm, tn);
+    }
+  };
   const int64_t split_tokens =
       ((p.M + p.splits - 1) / p.splits + C::kBK - 1) / C::kBK * C::kBK;  // a multiple of kBK
-  auto unit_of = [&](int u, int &e, int &tm, int &tn, int &sp, int32_t &m0, int64_t &len) -> int {
-    if (GR) {
-      resolve_tile<GR, kSgradGroup>(p, u, e, tm, tn);
-      sp = 0;
-      m0 = 0;
-      len = group_rows(p, e);
-      return static_cast<int>((len + C::kBK - 1) / C::kBK);
-    }
-    sp = p.splits > 1 ? u / tiles_per_split : 0;
-    resolve_tile<GR, kSgradGroup>(p, u - sp * tiles_per_split, e, tm, tn);
-    const int64_t first = static_cast<int64_t>(sp) * split_tokens;
-    len = p.M - first < split_tokens ? p.M - first : split_tokens;
+  auto tokens_of = [&](const Unit &w, int32_t &m0) -> int64_t {
+    m0 = 0;
+    if (GR) return w.e < cached ? s_rows[w.e] : group_rows(p, w.e);
+    const int64_t first = static_cast<int64_t>(w.e) * split_tokens;
     m0 = static_cast<int32_t>(first);
-    return len > 0 ? static_cast<int>((len + C::kBK - 1) / C::kBK) : 0;
+    return p.M - first < split_tokens ? (p.M - first > 0 ? p.M - first : 0) : split_tokens;
   };
 
   auto stage_a = [&](int s) { return smem + s * C::kStageBytes; };
@@ -1454,6 +1492,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(SgradPairCfg::kThrea
       mbar_init(&tfull[b], 1);
       mbar_init(&tempty[b], C::kEpiWarps);
     }
+    mbar_init(cfull, 1);
+    mbar_init(cempty, C::kEpiWarps);
     mbar_init(drain, 1);
     *abort_flag = 0;
     fence_barrier_init();
@@ -1462,7 +1502,19 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(SgradPairCfg::kThrea
   if (!GR && warp == C::kTmaWarp && lane == 0) {
     tma_prefetch_desc(&tmA);
     tma_prefetch_desc(&tmB);
+    tma_prefetch_desc(&tmC);
   }
+  for (int x = threadIdx.x; x < cached; x += C::kThreads) {
+    s_rows[x] = group_rows(p, x);
+    s_ids[x] = group_id(p, x);
+  }
+  for (int x = threadIdx.x; x < min(per, C::kCached); x += C::kThreads) {
+    int tm, tn;
+    tile_coords<kSgradGroup>(x, p.tiles_m, p.tiles_n, tm, tn);
+    s_tiles[x] = tn << 16 | tm;
+  }
+  Unit unit{cluster / per, cluster % per};
+  const Unit stride{nclusters / per, nclusters % per};
   tc_fence_before();
   cluster_sync_all();
   tc_fence_after();
@@ -1473,13 +1525,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(SgradPairCfg::kThrea
     if (lane == 0) {
       int it = 0;
       bool ok = true;
-      int e = 0, e_seen = -1;
+      int e_seen = -1;
       const CUtensorMap *mA = &tmA, *mB = &tmB;
-      for (int tile = cluster; tile < total && ok; tile += nclusters) {
-        int tm, tn, sp;
+      for (int tile = cluster; tile < total && ok; tile += nclusters, advance(unit, stride)) {
+        int tm, tn;
         int32_t m0;
-        int64_t len;
-        const int num_k = unit_of(tile, e, tm, tn, sp, m0, len);
+        tile_of(unit.local, tm, tn);
+        const int e = unit.e, num_k = static_cast<int>((tokens_of(unit, m0) + C::kBK - 1) / C::kBK);
         if (GR && e != e_seen && num_k > 0) {  // the expert's own token rows of dY and X (an expert
           mA = &group_maps(p, e)->m[0];        // without tokens has no descriptors and loads nothing)
           mB = &group_maps(p, e)->m[1];
@@ -1515,12 +1567,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(SgradPairCfg::kThrea
       uint32_t ph = 0;
       int tc = 0;
       bool ok = true;
-      int e = 0;
-      for (int tile = cluster; tile < total && ok; tile += nclusters, ++tc) {
-        int tm, tn, sp;
+      for (int tile = cluster; tile < total && ok; tile += nclusters, advance(unit, stride), ++tc) {
         int32_t m0;
-        int64_t len;
-        const int num_k = unit_of(tile, e, tm, tn, sp, m0, len);
+        const int64_t len = tokens_of(unit, m0);
+        const int num_k = static_cast<int>((len + C::kBK - 1) / C::kBK);
         // MMAs of 16 tokens in the last stage: the rest of it is past the unit's tokens
         const int last = num_k > 0 ? static_cast<int>((len - static_cast<int64_t>(num_k - 1) * C::kBK + 15) / 16) : 0;
         const int ab = tc & 1;
@@ -1554,67 +1604,108 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(SgradPairCfg::kThrea
       umma_commit_pair(drain);
       mbar_drain(drain, 0);
     }
+  } else if (warp == C::kCodeWarp) {
+    // ------------------------------------------------------ codes of the unit (both CTAs)
+    // One slot: the epilogue warps take their rows into registers at the start of a unit and
+    // it is filled again while they work on it.
+    if (FMT != kFmtBf16Mul && lane == 0) {
+      int tc = 0;
+      for (int tile = cluster; tile < total; tile += nclusters, advance(unit, stride), ++tc) {
+        int tm, tn;
+        tile_of(unit.local, tm, tn);
+        const int64_t eid = GR ? (unit.e < cached ? s_ids[unit.e] : group_id(p, unit.e)) : 0;  // expert of the entry
+        const int32_t y = static_cast<int32_t>(eid * p.N) + tm * C::kTile + 128 * static_cast<int32_t>(rank);
+        if (tc > 0 && !mbar_wait(cempty, (tc - 1) & 1, abort_flag, p.err)) break;
+        mbar_arrive_expect_tx(cfull, C::kCodes);
+        for (int j = 0; j < 2; ++j)
+          tma_load_2d(smem_u32(s_codes) + j * (C::kCodes / 2), &tmC, cfull, tn * (C::kTile / 2) + 64 * j, y);
+      }
+      if (*abort_flag && tc > 0) mbar_drain(cfull, (tc - 1) & 1);
+    }
   } else if (warp < C::kEpiWarps) {
-    // ------------------------------------------------------ epilogue (warps 0-7, both CTAs)
-    constexpr int kCols = C::kTile / 2;   // columns of a warp
+    // ------------------------------------------------------ epilogue (warps 0-15, both CTAs)
+    constexpr int kCols = C::kTile / 4;   // columns of a warp
     constexpr int kGroups = kCols / 32;   // 32-column groups of a warp
     constexpr int kPer = 32 / B;          // blocks of a group
-    const int quad = warp & 3, half = warp >> 2;
-    const uint32_t t_row = tmem_base + (static_cast<uint32_t>(quad * 32) << 16) + half * kCols;
-    const int64_t G = p.K / B;
-    // What this lane needs of a unit besides the accumulator: its row's packed codes and
-    // mask bytes (one group's bytes in one word), and where its gradient blocks go. The
-    // expert's code plane (the multiplicative control: its bf16 weights), gradient plane
-    // and mask; a token split writes its own partial plane, masked when the parts are added.
+    constexpr int kOut = kGroups * kPer;  // blocks of a row
+    const int quad = warp & 3, part_col = warp >> 2, row = quad * 32 + lane;
+    const uint32_t t_row = tmem_base + (static_cast<uint32_t>(quad * 32) << 16) + part_col * kCols;
+    const int64_t G = p.K / B, plane = p.N * G;
+    // the row's 32 code bytes of the 64 columns: two 16-byte chunks, 64-byte swizzle
+    const uint8_t *c_row = s_codes + (part_col >> 1) * (C::kCodes / 2) + row * 64;
+    const int chunk = 2 * (part_col & 1), swz = (row >> 1) & 3;
+    // What a unit needs besides the accumulator and the codes, fetched a unit ahead: its mask
+    // bytes (as loaded: any arithmetic on them there would wait for memory) and where its
+    // gradient blocks lie. A lane's row lies in lines of its own, so every load of the warp
+    // is 32 requests to the L1: one word of mask where its alignment allows, else bytes. A
+    // token split writes its own partial plane, masked when the parts are added.
+    const uint8_t *masks = p.splits > 1 ? nullptr : p.mask;
+    const bool wide_mask = G % kOut == 0 && reinterpret_cast<uintptr_t>(masks) % kOut == 0;
     struct Row {
-      uint4 cw[kGroups];
-      uint32_t mk[kGroups];
-      float *g;          // the row's block of column k
-      int64_t k;         // first column of this warp
-      const uint8_t *w;  // the row's bf16 weights (control)
-      bool live, empty_sum;
+      uint32_t mk[kOut];
+      int64_t b0;      // block of the row's first column among those of all planes
+      int left;        // columns from there, none: not a row of the unit
+      int part;        // token part
+      bool empty_sum;  // no tokens: the accumulator is never written
     };
-    int e = 0;
-    auto fetch = [&](int unit, Row &q) {
-      q.live = false;
-      if (unit >= total) return;
-      int tm, tn, sp;
+    // block of this lane's row and first column in tile (0, 0)
+    const int64_t lane_b = static_cast<int64_t>(128 * rank + row) * G + part_col * kOut;
+    float *const grads = p.splits > 1 ? p.partial : static_cast<float *>(p.out);
+    auto fetch = [&](bool in, Row &q) {
+      q.left = 0;
+      if (!in) return;
+      int tm, tn;
       int32_t m0;
-      int64_t len;
-      q.empty_sum = unit_of(unit, e, tm, tn, sp, m0, len) == 0;  // no tokens: the accumulator is never written
-      const int64_t eid = GR ? group_id(p, e) : 0;  // the expert of table entry e
-      const int64_t n = static_cast<int64_t>(tm) * C::kTile + 128 * rank + quad * 32 + lane;
-      q.k = static_cast<int64_t>(tn) * C::kTile + half * kCols;
-      q.live = n < p.N;
-      if (!q.live) return;
-      const int64_t b0 = n * G + q.k / B;
-      q.g = (p.splits > 1 ? p.partial + sp * p.N * G : static_cast<float *>(p.out) + (GR ? eid * p.N * G : 0)) + b0;
-      if (FMT == kFmtBf16Mul) q.w = p.codes + (n * p.K + q.k) * 2;
-      const uint8_t *codes = (GR ? p.codes + eid * p.N * (p.K / 2) : p.codes) + n * (p.K / 2) + q.k / 2;
-      const uint8_t *mask = p.mask && p.splits == 1 ? p.mask + (GR ? eid * p.N * G : 0) + b0 : nullptr;
+      tile_of(unit.local, tm, tn);
+      q.empty_sum = tokens_of(unit, m0) <= 0;
+      const int k = tn * C::kTile + part_col * kCols;
+      if (tm * C::kTile + static_cast<int>(128 * rank) + row >= p.N || k >= p.K) return;
+      q.left = static_cast<int>(p.K) - k;
+      const int64_t eid = GR ? (unit.e < cached ? s_ids[unit.e] : group_id(p, unit.e)) : 0;  // expert of the entry
+      q.part = GR ? 0 : unit.e;
+      q.b0 = eid * plane + static_cast<int64_t>(tm) * (C::kTile * G) + tn * (C::kTile / B) + lane_b;
+      const uint8_t *mask = masks + q.b0;
+      if (!masks) {
 #pragma unroll
-      for (int j = 0; j < kGroups; ++j) {
-        const bool in = q.k + 32 * j < p.K;
-        if (FMT != kFmtBf16Mul) q.cw[j] = in ? __ldg(reinterpret_cast<const uint4 *>(codes) + j) : make_uint4(0, 0, 0, 0);
-        q.mk[j] = 0x0101u;
-        if (mask && in) {  // byte loads: a mask may start at any address
-          q.mk[j] = __ldg(mask + kPer * j);
-          if (kPer == 2) q.mk[j] |= static_cast<uint32_t>(__ldg(mask + 2 * j + 1)) << 8;
+        for (int i = 0; i < kOut; ++i) q.mk[i] = wide_mask ? 0x01010101u : 1u;
+      } else if (wide_mask) {
+        q.mk[0] = kOut == 4 ? __ldg(reinterpret_cast<const uint32_t *>(mask))
+                            : __ldg(reinterpret_cast<const unsigned short *>(mask));
+      } else {  // bytes: a mask may start at any address
+#pragma unroll
+        for (int i = 0; i < kOut; ++i) {
+          q.mk[i] = 0;
+          if (B * i < q.left) q.mk[i] = __ldg(mask + i);
         }
       }
     };
     Row cur, next;
-    fetch(cluster, cur);
+    fetch(cluster < total, cur);
     int tc = 0;
     for (int tile = cluster; tile < total; tile += nclusters, ++tc) {
-      fetch(tile + nclusters, next);
+      advance(unit, stride);
+      fetch(tile + nclusters < total, next);
+      uint4 cw[kGroups];
+      if (FMT != kFmtBf16Mul) {
+        if (!mbar_wait(cfull, tc & 1, abort_flag, p.err)) break;
+#pragma unroll
+        for (int j = 0; j < kGroups; ++j) cw[j] = *reinterpret_cast<const uint4 *>(c_row + (((chunk + j) ^ swz) << 4));
+        // The slot may be written again only after these loads have returned, and nothing
+        // uses their results until much later: the vote waits for them (any lane may arrive).
+        const bool any = __any_sync(0xFFFFFFFFu, (cw[0].x ^ cw[kGroups - 1].x) == 1u);
+        __syncwarp();
+        if (lane == (any ? 1 : 0)) mbar_arrive(cempty);
+      }
       const int ab = tc & 1;
       const uint32_t au = static_cast<uint32_t>(tc >> 1);
       if (!mbar_wait(&tfull[ab], au & 1u, abort_flag, p.err)) break;
       tc_fence_after();
       const uint32_t t_buf = t_row + ab * kTmemCols;
+      auto mask_of = [&](int i) {
+        return static_cast<float>(wide_mask ? (cur.mk[0] >> (8 * i)) & 0xFFu : cur.mk[i]);
+      };
       uint32_t v[2][32];
-      float out[kGroups * kPer];
+      float out[kOut];
       tmem_ld32(t_buf, v[0]);
 #pragma unroll
       for (int j = 0; j < kGroups; ++j) {
@@ -1638,14 +1729,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(SgradPairCfg::kThrea
             }
           }
         }
-        const uint32_t words[4] = {cur.cw[j].x, cur.cw[j].y, cur.cw[j].z, cur.cw[j].w};
+        const uint32_t words[4] = {cw[j].x, cw[j].y, cw[j].z, cw[j].w};
         float part[4];
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
           uint32_t o[4];  // 8 weights of the row as bf16 pairs: decoded codes, or the control's bf16 W
           if (FMT == kFmtBf16Mul) {
             uint4 wq = make_uint4(0, 0, 0, 0);
-            if (cur.live && cur.k + 32 * j < p.K) wq = __ldg(reinterpret_cast<const uint4 *>(cur.w) + 4 * j + c);
+            if (32 * j < cur.left) wq = __ldg(reinterpret_cast<const uint4 *>(p.codes + cur.b0 * (2 * B)) + 4 * j + c);
             o[0] = wq.x;
             o[1] = wq.y;
             o[2] = wq.z;
@@ -1660,29 +1751,30 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(SgradPairCfg::kThrea
           part[c] = sum_f32x2(acc);
         }
         if (kPer == 2) {
-          out[2 * j] = (part[0] + part[1]) * static_cast<float>(cur.mk[j] & 0xFFu);
-          out[2 * j + 1] = (part[2] + part[3]) * static_cast<float>(cur.mk[j] >> 8);
+          out[2 * j] = (part[0] + part[1]) * mask_of(2 * j);
+          out[2 * j + 1] = (part[2] + part[3]) * mask_of(2 * j + 1);
         } else {
-          out[j] = ((part[0] + part[1]) + (part[2] + part[3])) * static_cast<float>(cur.mk[j] & 0xFFu);
+          out[j] = ((part[0] + part[1]) + (part[2] + part[3])) * mask_of(j);
         }
       }
-      if (cur.live) {
+      if (cur.left > 0) {
+        float *g = grads + cur.part * plane + cur.b0;
 #pragma unroll
-        for (int i = 0; i < kGroups * kPer; ++i) out[i] = cur.empty_sum ? 0.f : out[i];
-        // the warp's blocks of a row are contiguous: 16-byte stores where rows keep the
-        // alignment (plane pointers are 16-byte aligned, the first block a multiple of 4)
-        if ((G & 3) == 0 && cur.k + kCols <= p.K) {
-#pragma unroll
-          for (int i = 0; i < kGroups * kPer; i += 4)
-            *reinterpret_cast<float4 *>(cur.g + i) = make_float4(out[i], out[i + 1], out[i + 2], out[i + 3]);
+        for (int i = 0; i < kOut; ++i) out[i] = cur.empty_sum ? 0.f : out[i];
+        // the warp's blocks of a row are contiguous: one store where rows keep the alignment
+        // (plane pointers are 16-byte aligned, the first block a multiple of the blocks)
+        if (kPer == 2 && (G & 3) == 0 && kCols <= cur.left) {
+          *reinterpret_cast<float4 *>(g) = make_float4(out[0], out[1], out[kOut - 2], out[kOut - 1]);
+        } else if (kPer == 1 && (G & 1) == 0 && kCols <= cur.left) {
+          *reinterpret_cast<float2 *>(g) = make_float2(out[0], out[1]);
         } else {
 #pragma unroll
           for (int j = 0; j < kGroups; ++j) {
-            if (cur.k + 32 * j >= p.K) break;
+            if (32 * j >= cur.left) break;
             if (kPer == 2)
-              *reinterpret_cast<float2 *>(cur.g + 2 * j) = make_float2(out[2 * j], out[2 * j + 1]);
+              *reinterpret_cast<float2 *>(g + 2 * j) = make_float2(out[2 * j], out[2 * j + 1]);
             else
-              cur.g[j] = out[j];
+              g[j] = out[j];
           }
         }
       }
@@ -1738,12 +1830,12 @@ cudaError_t launch_pair(const KParams &p, const CUtensorMap &tmA, const CUtensor
 }
 
 template <int FMT, bool GR>
-cudaError_t launch_sgrad(const KParams &p, const CUtensorMap &tmA, const CUtensorMap &tmB, int sm_count,
-                         cudaStream_t stream) {
+cudaError_t launch_sgrad(const KParams &p, const CUtensorMap &tmA, const CUtensorMap &tmB, const CUtensorMap &tmC,
+                         int sm_count, cudaStream_t stream) {
   static int done_mask = 0;
   static int max_clusters[32] = {0};
   return launch_persistent(sq_sgrad_pair_kernel<FMT, GR>, SgradPairCfg::kThreads, SgradPairCfg::kSmemBytes, p.total,
-                           sm_count, stream, max_clusters, &done_mask, tmA, tmB, p);
+                           sm_count, stream, max_clusters, &done_mask, tmA, tmB, tmC, p);
 }
 
 }  // namespace

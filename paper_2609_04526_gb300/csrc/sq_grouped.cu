@@ -17,11 +17,11 @@ cudaError_t launch_grouped(const GroupedArgs &a, const CUtensorMap &tmCodes, int
   if (a.fmt == 0) {
     if (a.mode == MODE_FWD) return launch_pair<MODE_FWD, 0, true>(p, tmCodes, tmCodes, tmCodes, sm_count, stream);
     if (a.mode == MODE_DX) return launch_pair<MODE_DX, 0, true>(p, tmCodes, tmCodes, tmCodes, sm_count, stream);
-    return launch_sgrad<0, true>(p, tmCodes, tmCodes, sm_count, stream);
+    return launch_sgrad<0, true>(p, tmCodes, tmCodes, tmCodes, sm_count, stream);
   }
   if (a.mode == MODE_FWD) return launch_pair<MODE_FWD, 1, true>(p, tmCodes, tmCodes, tmCodes, sm_count, stream);
   if (a.mode == MODE_DX) return launch_pair<MODE_DX, 1, true>(p, tmCodes, tmCodes, tmCodes, sm_count, stream);
-  return launch_sgrad<1, true>(p, tmCodes, tmCodes, sm_count, stream);
+  return launch_sgrad<1, true>(p, tmCodes, tmCodes, tmCodes, sm_count, stream);
 }
 
 }  // namespace sqi

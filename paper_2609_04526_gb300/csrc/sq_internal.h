@@ -219,7 +219,7 @@ struct GroupedArgs {
 };
 
 // Launch one grouped contraction. tmCodes is the descriptor of all experts'
-// packed codes as one [E * N, K/2] tensor (MODE_FWD / MODE_DX; unused for MODE_SGRAD).
+// packed codes as one [E * N, K/2] tensor.
 cudaError_t launch_grouped(const GroupedArgs &a, const CUtensorMap &tmCodes, int sm_count, cudaStream_t stream);
 
 // The contractions of the full-precision multiplicative control (a.fmt ignored):
@@ -236,9 +236,10 @@ cudaError_t launch_lowrank_product(int64_t N, int64_t G, int r, float alpha_over
 
 // Launch one contraction. tmA is the TMA descriptor of the streamed bf16
 // activations; tmB that of the packed codes (MODE_FWD / MODE_DX) or of the second
-// bf16 operand (MODE_SGRAD); tmOut that of the bf16 output (MODE_FWD / MODE_DX:
-// 32-row x 32-column boxes, 64-byte swizzle; null for MODE_SGRAD).
-cudaError_t launch_gemm(const GemmArgs &a, const CUtensorMap &tmA, const CUtensorMap &tmB, const CUtensorMap *tmOut,
+// bf16 operand (MODE_SGRAD); tmC that of the bf16 output (MODE_FWD / MODE_DX:
+// 32-row x 32-column boxes, 64-byte swizzle) or of the packed codes (MODE_SGRAD). Codes
+// come in boxes of 64 bytes x 128 rows, 64-byte swizzle.
+cudaError_t launch_gemm(const GemmArgs &a, const CUtensorMap &tmA, const CUtensorMap &tmB, const CUtensorMap &tmC,
                         int sm_count, cudaStream_t stream);
 // One thread waiting on a barrier nothing arrives on, bounded like every kernel wait:
 // records kErrWaitTimeout in *err and returns (the failure-path self-test).

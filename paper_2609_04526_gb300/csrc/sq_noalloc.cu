@@ -94,6 +94,17 @@ bool encode_act(CUtensorMap *map, const void *ptr, int64_t inner, int64_t outer)
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Packed codes [N, K/2] in 64-byte x 128-row boxes with the 64-byte swizzle.
+bool encode_codes(CUtensorMap *map, const uint8_t *ptr, int64_t K2, int64_t N) {
+  const cuuint64_t dims[2] = {static_cast<cuuint64_t>(K2), static_cast<cuuint64_t>(N)};
+  const cuuint64_t strides[1] = {static_cast<cuuint64_t>(K2)};
+  const cuuint32_t box[2] = {64, 128};
+  const cuuint32_t estr[2] = {1, 1};
+  return g_encode(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<uint8_t *>(ptr), dims, strides, box, estr,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 }  // namespace
 
 extern "C" sq_status sq_scale_grad_noalloc(const sq_weight *w, const uint16_t *X, const uint16_t *dY, int64_t M,
@@ -123,8 +134,10 @@ extern "C" sq_status sq_scale_grad_noalloc(const sq_weight *w, const uint16_t *X
     if (cudaMemsetAsync(g, 0, static_cast<size_t>(w->N) * (w->K / B) * sizeof(float), s) != cudaSuccess)
       return SQ_ERR_CUDA;
   } else {
-    CUtensorMap tmA, tmB;
-    if (!encode_act(&tmA, dY, w->N, M) || !encode_act(&tmB, X, w->K, M)) return SQ_ERR_CUDA;
+    CUtensorMap tmA, tmB, tmC;
+    if (!encode_act(&tmA, dY, w->N, M) || !encode_act(&tmB, X, w->K, M) ||
+        !encode_codes(&tmC, w->codes, w->K / 2, w->N))
+      return SQ_ERR_CUDA;
     sqi::GemmArgs a;
     a.mode = sqi::MODE_SGRAD;
     a.fmt = w->fmt;
@@ -137,7 +150,7 @@ extern "C" sq_status sq_scale_grad_noalloc(const sq_weight *w, const uint16_t *X
     a.out = g;
     a.mask = mask;
     a.err = scratch;
-    if (sqi::launch_gemm(a, tmA, tmB, nullptr, dev->sm_count, s) != cudaSuccess) return SQ_ERR_CUDA;
+    if (sqi::launch_gemm(a, tmA, tmB, tmC, dev->sm_count, s) != cudaSuccess) return SQ_ERR_CUDA;
   }
   if (device_status &&
       cudaMemcpyAsync(device_status, scratch, sizeof(int32_t), cudaMemcpyDeviceToDevice, s) != cudaSuccess)

@@ -35,6 +35,63 @@ def test_scale_gradient_of_few_tokens(fmt, M):
 
 
 @pytest.mark.parametrize("fmt", [0, 1])
+@pytest.mark.parametrize("N,K", [(264, 512), (136, 96), (40, 288)])
+def test_scale_gradient_masks_at_any_address(fmt, N, K):
+    """The mask is read in words where its address and its rows allow and in bytes elsewhere:
+    at every address the gradient is the unmasked one times the mask, bit for bit."""
+    import paper_2609_04526_gb300 as pkg
+    from paper_2609_04526_gb300 import synth
+    h = pkg.Handle()
+    wl = synth.custom("few", fmt, 50, N, K, seed=N + K)
+    w, X, dY = setup_linear(wl, wl.linears[0])
+    G = K // wl.block
+    full = h.sq_scale_grad(w, X, dY)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(K)
+    bits = torch.rand(N, G, generator=gen, device="cuda") < 0.7
+    for start in range(5):
+        store = torch.full((N * G + 5,), 7, dtype=torch.uint8, device="cuda")
+        mask = store[start:start + N * G].view(N, G)
+        mask.copy_(bits)
+        g = h.sq_scale_grad(w, X, dY, mask=mask)
+        h.sq_sync()
+        assert torch.equal(g, full * bits), start
+
+
+@pytest.mark.parametrize("fmt", [0, 1])
+def test_scale_gradient_beyond_the_tables(fmt):
+    """More experts than the kernel keeps in shared memory, and a weight of more tiles."""
+    import paper_2609_04526_gb300 as pkg
+    from paper_2609_04526_gb300 import synth
+    h = pkg.Handle()
+    E, N, K = 1100, 16, 64
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(fmt)
+    codes = torch.randint(0, 256, (E, N, K // 2), generator=gen, device="cuda", dtype=torch.uint8)
+    scales = torch.full((E, N, K // (16 if fmt == 0 else 32)), 0x38, dtype=torch.uint8, device="cuda")
+    gw = pkg.GroupedWeight(fmt, E, N, K, codes, scales, [1.0] * E)
+    off = [0]
+    for e in range(E):
+        off.append(off[-1] + e % 4)
+    X = torch.randn(off[-1], K, generator=gen, device="cuda").bfloat16()
+    dY = torch.randn(off[-1], N, generator=gen, device="cuda").bfloat16()
+    g = h.sq_grouped_scale_grad(gw, off, X, dY)
+    h.sq_sync()
+    for e in (0, 1, 2, 3, 1023, 1024, 1025, 1027, 1098, 1099):
+        a, b = off[e], off[e + 1]
+        ref = oracle.scale_grad(fmt, host(codes[e]), hbits(X[a:b]), hbits(dY[a:b]))
+        assert_close(f64(g[e]), ref, what=f"g of expert {e}")
+
+    wl = synth.custom("few", fmt, 20, 8712, 8224, seed=fmt)   # 35 x 33 tiles
+    w, X, dY = setup_linear(wl, wl.linears[0])
+    g = h.sq_scale_grad(w, X, dY)
+    h.sq_sync()
+    rows = np.array([0, 255, 256, 4095, 4096, 7935, 7936, 8191, 8192, 8447, 8448, 8711])
+    ref = oracle.scale_grad(fmt, host(w.codes), hbits(X), hbits(dY), rows=rows)
+    assert_close(f64(g)[rows], ref, what="g of a large weight")
+
+
+@pytest.mark.parametrize("fmt", [0, 1])
 @pytest.mark.parametrize("M,N,K", [
     (1, 8, 32),          # one MMA step of everything
     (16, 120, 160), (17, 136, 96),   # a feature tile's edge, half a stage of the contraction
