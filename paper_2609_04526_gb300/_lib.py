@@ -164,16 +164,22 @@ def _offsets(offsets, E: int):
     return (ctypes.c_int64 * len(vals))(*vals), vals
 
 
+# Pointers and streams go to the library as plain integers: its argument and structure
+# types (c_void_p) take them without a wrapper object.
 def _ptr(t: Optional[torch.Tensor]):
     if t is None:
         return None
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
-def _stream(stream) -> ctypes.c_void_p:
+def _stream(stream) -> int:
+    """The caller's stream, or the current one of the current device. torch.cuda.current_stream()
+    builds a Stream object, 3.1 us of a call whose library part is 2.8 us; the raw handle is 0.2 us."""
     if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
+        if torch.cuda.is_initialized():
+            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+        stream = torch.cuda.current_stream()  # initialises CUDA, or raises where there is none
+    return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
 class Handle:
