@@ -326,7 +326,7 @@ __global__ void __launch_bounds__(32 * (WARPS + 2), 16 / WARPS)
     bool ok = true;
     int s = grp;  // ring slot and use parity of the group's stage (GROUPS <= stages)
     uint32_t ph = 0;
-    int cs = grp / kPer;  // code slot and its use parity
+    int cs = grp / kPer;  // code slot and its use parity (few_ring: which slot counts this can follow)
     uint32_t cph = 0;
     while (cs >= p.slots) {
       cs -= p.slots;
@@ -475,9 +475,8 @@ cudaError_t launch_few(const FewArgs &a, const CUtensorMap (&tmX)[3], const CUte
   p.slots = ring.slots;
   for (p.tmem_cols = 32; p.tmem_cols < a.tile_tokens; p.tmem_cols *= 2) {
   }
-  if (ring.depth == 128) return launch_shape<128, 16, 2>(a, p, maps, ring.bytes, stream);
-  return ring.stages >= 4 ? launch_shape<64, 8, 4>(a, p, maps, ring.bytes, stream)
-                          : launch_shape<64, 8, 2>(a, p, maps, ring.bytes, stream);
+  return ring.depth == 128 ? launch_shape<128, 16, kFewGroups>(a, p, maps, ring.bytes, stream)
+                           : launch_shape<64, 8, kFewGroups>(a, p, maps, ring.bytes, stream);
 }
 
 }  // namespace sqi

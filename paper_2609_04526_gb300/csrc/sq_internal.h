@@ -100,7 +100,8 @@ constexpr int kFewBoxRows = 32;        // tokens of the smallest TMA box
 constexpr int kFewSmemBytes = 111 * 1024;  // of a CTA: two share an SM
 constexpr int kFewSmemAlone = 224 * 1024;  // ... where the launch has at most one CTA per SM
 constexpr int kFewSlotBytes = 128 * 64;    // packed codes of 128 x 128 weights
-constexpr int kFewMaxStages = 4, kFewMaxSlots = 12;
+constexpr int kFewMaxStages = 3, kFewMaxSlots = 12;
+constexpr int kFewGroups = 2;              // sets of decode warps, which take the stages in turn
 
 // Tokens of the equal tiles (whole MMA steps of 16) that `rows` tokens are cut into.
 inline int few_tile_tokens(int64_t rows, int limit) {
@@ -115,6 +116,13 @@ inline int few_box_rows(int tile_tokens) {
 // Shared memory of a CTA: `stages` stages of `depth` contraction indices (decoded weights
 // and activations) and `slots` code slots, so the codes run ahead of the MMAs by the slots
 // less the stages' share of them. The epilogue's bf16 tile reuses the stages.
+//
+// A code slot holds 128 / depth stages, and a set of decode warps waits by parity for the
+// slot of its next stage. That wait can only be told from one for an earlier use of the slot
+// if the use before is known to have landed: because the same set read it (a slot's uses lie
+// slots * 128 / depth stages apart), or because its MMAs are done (a set that starts on stage
+// i has seen those of stage i - kFewGroups - stages). A slot count that gives neither loses
+// one. (Four stages, three slots and four sets for up to 32 tokens gave neither.)
 struct FewRing {
   int depth, stage_bytes, stages, slots;
   int bytes;  // with 1 KiB for the alignment
@@ -128,9 +136,11 @@ inline FewRing few_ring(int tile_tokens, bool alone) {
   if (alone)
     r.stages = rows <= 96 ? 3 : 2;
   else
-    r.stages = rows <= 32 ? 4 : rows <= 64 ? 3 : 2;
+    r.stages = rows <= 64 ? 3 : 2;
   r.slots = (room - r.stages * r.stage_bytes) / kFewSlotBytes;
   if (r.slots > kFewMaxSlots) r.slots = kFewMaxSlots;
+  const int reuse = r.slots * (128 / r.depth);
+  if (reuse % kFewGroups != 0 && reuse < kFewGroups + r.stages) --r.slots;
   r.bytes = r.stages * r.stage_bytes + r.slots * kFewSlotBytes + 1024;
   return r;
 }

@@ -72,11 +72,14 @@ def test_every_plan_fits(plan):
         assert few < 0.97 * pair
         assert tokens % 16 == 0 and 16 <= tokens <= limit <= 256 and (tokens <= 192 or alone)
         assert depth == (128 if alone else 64) and stage == (128 + math.ceil(tokens / 32) * 32) * depth * 2
-        assert stages >= (2 if depth == 128 else 2) and stages <= 4 and 2 <= slots <= 12
+        assert 2 <= stages <= 3 and 2 <= slots <= 12
         assert nbytes == stages * stage + slots * 8192 + 1024
         # shared memory of a CTA (227 KiB less the static part), or of two on an SM (228 KiB less 1 KiB each)
         assert nbytes + 512 <= 227 * 1024 if alone else 2 * (nbytes + 512 + 1024) <= 228 * 1024
         assert tokens * 256 <= nbytes - 1024  # the epilogue's bf16 tile
+        # a set of decode warps (of two) can tell its use of a code slot from the use before
+        reuse = slots * 128 / depth
+        assert reuse % 2 == 0 or reuse >= 2 + stages
         # the codes run ahead of the stages in flight
         assert slots >= math.ceil(stages * depth / 128) + (0 if depth == 128 and stages == 2 else 1)
     assert chosen > 500
