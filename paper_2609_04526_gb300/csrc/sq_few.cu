@@ -17,12 +17,15 @@
 //   64-deep stages, 8 decode warps, two CTAs per SM, so that one computes while the other
 //   starts up, waits for memory or drains: larger launches.
 //
-// Measured (forward; before: the pair kernel): 4096 x 4096 at 187 tokens 43 -> 25 us, 1024 x
+// Measured (forward; before: the pair kernel): 4096 x 4096 at 187 tokens 43 -> 22.6 us, 1024 x
 // 4096 at 2048 tokens 44 -> 25 us, 128 experts of 768 x 2048 with 128 rows each 131 -> 87 us,
 // of 2880 x 2880 with 16 rows each 566 -> 271 us (2.1 TB/s of codes). clock64 traces of one
 // CTA show its pace set by the decode warps' issue slots and by the MMA and TMA warps' own
 // instructions beside them (a barrier test ~110 cycles, a commit ~100, a TMA load ~150), not
 // by the tensor core or the memory: hence the long stages, and one elected lane per warp.
+// Codes and activations have a TMA warp each: with one for both a stage of a CTA alone took
+// 0.60 us where it takes 0.54 (4096 x 4096 at 187 tokens 24.7 -> 22.6 us, 4096 x 14336 at 64
+// tokens 71.9 -> 61.6 us; the experts' launches, two CTAs per SM, are unchanged).
 // Codes loaded by the decode warps into registers, four units ahead, were 20-50 % slower and
 // the experts' forward half as fast; 64-deep stages took 29-33 us for the 25 us launches.
 #include <climits>
@@ -84,10 +87,10 @@ __device__ __forceinline__ void tma_load_2d_elect(uint32_t dst, const CUtensorMa
 // BK: contraction depth of a stage. WARPS: decode warps, which then run the epilogue.
 // GROUPS: see the decode warps.
 template <int MODE, int FMT, int BK, int WARPS, int GROUPS>
-__global__ void __launch_bounds__(32 * (WARPS + 2), 16 / WARPS)
+__global__ void __launch_bounds__(32 * (WARPS + 3), 16 / WARPS)
     sq_gemm_few_kernel(const __grid_constant__ FewMaps maps, const FewParams p) {
   using C = FewCfg;
-  constexpr int kTmaWarp = WARPS, kMmaWarp = WARPS + 1, kThreads = 32 * (WARPS + 2);
+  constexpr int kTmaWarp = WARPS, kMmaWarp = WARPS + 1, kCodeWarp = WARPS + 2, kThreads = 32 * (WARPS + 3);
   constexpr int kA = C::kF * BK * 2;                         // decoded weights of a stage
   constexpr int kUnits = 4 * BK * GROUPS / (32 * WARPS);     // 32-weight units of a thread per stage
   constexpr int kPer = 128 / BK;                             // stages of a code slot
@@ -125,20 +128,53 @@ __global__ void __launch_bounds__(32 * (WARPS + 2), 16 / WARPS)
   const int boxes = (tile.rows + C::kBoxRows - 1) / C::kBoxRows;
 
   uint8_t *code_ring = smem + S * p.stage_bytes;
-  // The TMA thread sets the barriers up and starts at once; the others meet it at `start`
-  // before they touch one.
+  // The two TMA warps set up the barriers they wait on and start at once; the others meet
+  // them at `start` before they touch one.
   auto start = [] { asm volatile("barrier.sync 1, %0;" ::"n"(kThreads) : "memory"); };
 
-  if (warp == kTmaWarp) {
-    // ------------------------------------------------------ packed codes and activations
+  if (warp == kCodeWarp) {
+    // ------------------------------------------------------ packed codes
+    // The whole warp walks the slots and an elected lane issues (see the MMA warp). A slot
+    // holds 128 rows x 64 bytes: FWD 128 feature rows x 128 k, DX 128 contraction rows x
+    // 128 feature columns.
+    if (lane == 0) {
+      for (int c = 0; c < p.slots; ++c) {
+        mbar_init(&cfull[c], 1);
+        mbar_init(&cempty[c], kPer * (WARPS / GROUPS));
+      }
+      abort_word = 0;
+      fence_barrier_init();
+      fence_proxy_async_smem();
+    }
+    __syncwarp();
+    asm volatile("barrier.arrive 1, %0;" ::"n"(kThreads) : "memory");
+    const int fills = (cnt + kPer - 1) / kPer;
+    const int cx = MODE == MODE_FWD ? 0 : static_cast<int>(f0 / 2);
+    const int cy = static_cast<int>(tile.expert * p.N) + (MODE == MODE_FWD ? static_cast<int>(f0) : 0);
+    int j = 0, c = 0;  // slots filled, the next one and its use parity
+    uint32_t ph = 0;
+    for (; j < fills; ++j) {
+      if (j >= p.slots && !__all_sync(0xFFFFFFFFu, mbar_wait(&cempty[c], ph ^ 1u, abort_flag, p.err))) break;
+      expect_tx_elect(&cfull[c], C::kC);
+      tma_load_2d_elect(smem_u32(code_ring) + c * C::kC, &maps.codes, &cfull[c], cx + (MODE == MODE_FWD ? j * 64 : 0),
+                        cy + (MODE == MODE_FWD ? 0 : j * 128));
+      if (++c == p.slots) {
+        c = 0;
+        ph ^= 1u;
+      }
+    }
+    // after an abort: wait, with a limit, for the copies in flight
+    if (*abort_flag) {
+      for (int i = (j > p.slots ? j - p.slots : 0); i < j; ++i)
+        mbar_drain(&cfull[i % p.slots], static_cast<uint32_t>(i / p.slots) & 1u);
+    }
+    __syncwarp();
+  } else if (warp == kTmaWarp) {
+    // ------------------------------------------------------ activations
     if (lane == 0) {
       for (int s = 0; s < S; ++s) {
         mbar_init(&full[s], 1 + WARPS / GROUPS);
         mbar_init(&empty[s], 1);
-      }
-      for (int c = 0; c < p.slots; ++c) {
-        mbar_init(&cfull[c], 1);
-        mbar_init(&cempty[c], kPer * (WARPS / GROUPS));
       }
       mbar_init(done, 1);
       abort_word = 0;
@@ -147,33 +183,12 @@ __global__ void __launch_bounds__(32 * (WARPS + 2), 16 / WARPS)
     }
     __syncwarp();
     asm volatile("barrier.arrive 1, %0;" ::"n"(kThreads) : "memory");
-    // The whole warp walks the stages and an elected lane issues (see the MMA warp).
-    // A code slot holds 128 rows x 64 bytes: FWD 128 feature rows x 128 k, DX 128
-    // contraction rows x 128 feature columns.
-    const int fills = (cnt + kPer - 1) / kPer;
-    const int cx = MODE == MODE_FWD ? 0 : static_cast<int>(f0 / 2);
-    const int cy = static_cast<int>(tile.expert * p.N) + (MODE == MODE_FWD ? static_cast<int>(f0) : 0);
-    int j = 0, c = 0;  // code slots filled, the next one and its use parity
-    uint32_t cph = 0;
-    auto fill_codes = [&]() -> bool {
-      if (j >= p.slots && !__all_sync(0xFFFFFFFFu, mbar_wait(&cempty[c], cph ^ 1u, abort_flag, p.err))) return false;
-      expect_tx_elect(&cfull[c], C::kC);
-      tma_load_2d_elect(smem_u32(code_ring) + c * C::kC, &maps.codes, &cfull[c], cx + (MODE == MODE_FWD ? j * 64 : 0),
-                        cy + (MODE == MODE_FWD ? 0 : j * 128));
-      ++j;
-      if (++c == p.slots) {
-        c = 0;
-        cph ^= 1u;
-      }
-      return true;
-    };
-    bool ok = true;
     int it = 0, s = 0;
     uint32_t ph = 0, dst = smem_u32(smem) + kA;
     // Rows past the tile's last token (the next expert's, or zeros past M) only fill
     // accumulator columns that nothing stores.
-    auto fill_stage = [&]() -> bool {
-      if (it >= S && !__all_sync(0xFFFFFFFFu, mbar_wait(&empty[s], ph ^ 1u, abort_flag, p.err))) return false;
+    for (; it < cnt; ++it) {
+      if (it >= S && !__all_sync(0xFFFFFFFFu, mbar_wait(&empty[s], ph ^ 1u, abort_flag, p.err))) break;
       expect_tx_elect(&full[s], static_cast<uint32_t>((p.tiles ? boxes * C::kBoxRows : p.box_rows) * (BK * 2)));
 #pragma unroll
       for (int h = 0; h < BK / 64; ++h) {  // 64-wide chunks of the contraction
@@ -192,31 +207,16 @@ __global__ void __launch_bounds__(32 * (WARPS + 2), 16 / WARPS)
           if (boxes & 1) tma_load_2d_elect(d + b * C::kBox, &maps.box[0], &full[s], x, tile.row0 + b * C::kBoxRows);
         }
       }
-      ++it;
       dst += p.stage_bytes;
       if (++s == S) {
         s = 0;
         dst = smem_u32(smem) + kA;
         ph ^= 1u;
       }
-      return true;
-    };
-    ok = fill_codes() && fill_stage();
-    while (ok && j < fills && j < p.slots) ok = fill_codes();
-    while (ok && it < cnt) {
-      ok = fill_stage();
-      // the MMAs of stage it - 1 - S are done, so its codes are read: with a slot's last
-      // stage that slot is free, and this wait is over at once
-      if (ok && it > S && (it - S) % kPer == 0 && j < fills) ok = fill_codes();
     }
-    while (ok && j < fills) ok = fill_codes();
     // after an abort: wait, with a limit, for the copies in flight (an aborted stage may
     // never complete its other arrivals, so only for the last of those)
-    if (*abort_flag) {
-      for (int i = (j > p.slots ? j - p.slots : 0); i < j; ++i)
-        mbar_drain(&cfull[i % p.slots], static_cast<uint32_t>(i / p.slots) & 1u);
-      if (it > 0) mbar_drain(&full[(it - 1) % S], static_cast<uint32_t>((it - 1) / S) & 1u);
-    }
+    if (*abort_flag && it > 0) mbar_drain(&full[(it - 1) % S], static_cast<uint32_t>((it - 1) / S) & 1u);
     __syncwarp();
   } else if (warp == kMmaWarp) {
     // ------------------------------------------------------ MMA issuer
@@ -438,7 +438,7 @@ cudaError_t launch_one(const FewParams &p, const FewMaps &maps, int64_t units, i
       return e;
     done_mask |= 1 << (dev & 31);
   }
-  kernel<<<static_cast<unsigned>(units), 32 * (WARPS + 2), smem, stream>>>(maps, p);
+  kernel<<<static_cast<unsigned>(units), 32 * (WARPS + 3), smem, stream>>>(maps, p);
   return cudaGetLastError();
 }
 

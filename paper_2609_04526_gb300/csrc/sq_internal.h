@@ -164,18 +164,18 @@ struct FewArgs {
 // were fitted to measured launches (weights of 4096 x 4096, 1024 x 4096, 14336 x 4096, 768 x
 // 2048 and 256 x 512 at 16 to 4096 tokens; 128 experts of 768 x 2048 and 2880 x 2880 with 2 to
 // 1024 rows each) and lie within 20 % of them above 15 us. Both sides of the line, few-token
-// against pair kernel, in us: 4096 x 4096 25 against 43 at 16 to 512 tokens, 31 against 45 at
+// against pair kernel, in us: 4096 x 4096 23 against 43 at 16 to 192 tokens, 31 against 45 at
 // 1024, 78 against 45 at 2048; 1024 x 4096 25 against 44 at 2048; 768 x 2048 experts 77 against
 // 127 with 64 rows each, 139 against 148 with 256, 223 against 198 with 512; 2880 x 2880
 // experts 271 against 566 with 16 rows each, 345 against 520 with 128, 581 against 567 with 256.
 //
-// few_us, for token tiles of `tokens` tokens on average: a CTA alone on its SM takes 0.61 us
+// few_us, for token tiles of `tokens` tokens on average: a CTA alone on its SM takes 0.56 us
 // per 128-deep stage, more above 128 tokens (two stages in flight); CTAs that share an SM 0.27
 // us and up with the tokens per 64-deep stage, and 1.5 us to start and drain.
 inline double few_us(int64_t token_tiles, double tokens, int64_t features, int64_t contraction, int sm_count) {
   const int64_t ctas = token_tiles * ((features + kFewFeatures - 1) / kFewFeatures);
   if (ctas <= sm_count)
-    return 4.8 + ((contraction + 127) / 128) * (0.61 + (tokens > 128 ? 0.0015 * (tokens - 128) : 0.0));
+    return 4.8 + ((contraction + 127) / 128) * (0.56 + (tokens > 128 ? 0.0015 * (tokens - 128) : 0.0));
   const double per_sm = ctas > 4 * sm_count ? static_cast<double>(ctas) / sm_count
                                             : static_cast<double>((ctas + sm_count - 1) / sm_count);
   return 4.8 + per_sm * (((contraction + 63) / 64) * (0.27 + 0.0006 * tokens) + 1.5);
