@@ -278,7 +278,9 @@ sq_status run_few(sq_handle h, DeviceState *dev, int mode, int fmt, int E, int64
   f.err = dev->err_word;
   f.tiles = tiles;
   f.tile_tokens = tile_tokens;
-  f.units = token_tiles * (((mode == sqi::MODE_FWD ? N : K) + sqi::kFewFeatures - 1) / sqi::kFewFeatures);
+  const int64_t features = mode == sqi::MODE_FWD ? N : K;
+  f.features = sqi::few_features(token_tiles, tile_tokens, features, dev->sm_count);
+  f.units = token_tiles * ((features + f.features - 1) / f.features);
   const cudaError_t e = sqi::launch_few(f, tmX, tmCodes, dev->sm_count, stream);
   if (e != cudaSuccess) return cuda_fail(h, e, "few-token kernel launch");
   return SQ_OK;

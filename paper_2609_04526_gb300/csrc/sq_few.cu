@@ -12,12 +12,14 @@
 //
 // Three rings feed the MMA warp: packed codes (TMA, run far ahead: the first touches of a
 // weight take 2,000 to 3,000 cycles), activations (TMA) and the weights that the decode
-// warps make of the codes; the last two share stages. Two shapes:
-//   128-deep stages, 16 decode warps, one CTA per SM: launches of at most one CTA per SM.
+// warps make of the codes; the last two share stages. Three shapes:
+//   128-deep stages, 16 decode warps in two sets, one CTA per SM: launches of at most one
+//   CTA per SM.
+//   The same with 64 features and four sets: where twice as many tiles still have an SM each.
 //   64-deep stages, 8 decode warps, two CTAs per SM, so that one computes while the other
 //   starts up, waits for memory or drains: larger launches.
 //
-// Measured (forward; before: the pair kernel): 4096 x 4096 at 187 tokens 43 -> 22.6 us, 1024 x
+// Measured (forward; before: the pair kernel): 4096 x 4096 at 187 tokens 43 -> 18.5 us, 1024 x
 // 4096 at 2048 tokens 44 -> 25 us, 128 experts of 768 x 2048 with 128 rows each 131 -> 87 us,
 // of 2880 x 2880 with 16 rows each 566 -> 271 us (2.1 TB/s of codes). clock64 traces of one
 // CTA show its pace set by the decode warps' issue slots and by the MMA and TMA warps' own
@@ -25,7 +27,8 @@
 // by the tensor core or the memory: hence the long stages, and one elected lane per warp.
 // Codes and activations have a TMA warp each: with one for both a stage of a CTA alone took
 // 0.60 us where it takes 0.54 (4096 x 4096 at 187 tokens 24.7 -> 22.6 us, 4096 x 14336 at 64
-// tokens 71.9 -> 61.6 us; the experts' launches, two CTAs per SM, are unchanged).
+// tokens 71.9 -> 61.6 us; the experts' launches, two CTAs per SM, are unchanged); in tiles of
+// 64 features 0.43 us (18.5 and 46 us).
 // Codes loaded by the decode warps into registers, four units ahead, were 20-50 % slower and
 // the experts' forward half as fast; 64-deep stages took 29-33 us for the 25 us launches.
 #include <climits>
@@ -85,14 +88,15 @@ __device__ __forceinline__ void tma_load_2d_elect(uint32_t dst, const CUtensorMa
 }
 
 // BK: contraction depth of a stage. WARPS: decode warps, which then run the epilogue.
-// GROUPS: see the decode warps.
-template <int MODE, int FMT, int BK, int WARPS, int GROUPS>
+// GROUPS: see the decode warps. FEAT: output features of a tile; of 64 the MMAs' upper 64
+// rows multiply whatever the shared memory holds, into accumulator lanes that nothing reads.
+template <int MODE, int FMT, int BK, int WARPS, int GROUPS, int FEAT>
 __global__ void __launch_bounds__(32 * (WARPS + 3), 16 / WARPS)
     sq_gemm_few_kernel(const __grid_constant__ FewMaps maps, const FewParams p) {
   using C = FewCfg;
   constexpr int kTmaWarp = WARPS, kMmaWarp = WARPS + 1, kCodeWarp = WARPS + 2, kThreads = 32 * (WARPS + 3);
-  constexpr int kA = C::kF * BK * 2;                         // decoded weights of a stage
-  constexpr int kUnits = 4 * BK * GROUPS / (32 * WARPS);     // 32-weight units of a thread per stage
+  constexpr int kA = FEAT * BK * 2;                          // decoded weights of a stage
+  constexpr int kUnits = FEAT / 32 * BK * GROUPS / (32 * WARPS);  // 32-weight units of a thread per stage
   constexpr int kPer = 128 / BK;                             // stages of a code slot
   static_assert(GROUPS % kPer == 0 && C::kAhead % kUnits == 0, "a group's stages share one half of their slots");
   extern __shared__ uint8_t few_smem_raw[];
@@ -123,7 +127,7 @@ __global__ void __launch_bounds__(32 * (WARPS + 3), 16 / WARPS)
   }
   const int64_t F = MODE == MODE_FWD ? p.N : p.K;   // output features
   const int64_t Kc = MODE == MODE_FWD ? p.K : p.N;  // contraction
-  const int64_t f0 = static_cast<int64_t>(ft) * C::kF;
+  const int64_t f0 = static_cast<int64_t>(ft) * FEAT;
   const int cnt = static_cast<int>((Kc + BK - 1) / BK);  // stages
   const int boxes = (tile.rows + C::kBoxRows - 1) / C::kBoxRows;
 
@@ -136,7 +140,7 @@ __global__ void __launch_bounds__(32 * (WARPS + 3), 16 / WARPS)
     // ------------------------------------------------------ packed codes
     // The whole warp walks the slots and an elected lane issues (see the MMA warp). A slot
     // holds 128 rows x 64 bytes: FWD 128 feature rows x 128 k, DX 128 contraction rows x
-    // 128 feature columns.
+    // 128 feature columns (a tile of 64 features uses the first half).
     if (lane == 0) {
       for (int c = 0; c < p.slots; ++c) {
         mbar_init(&cfull[c], 1);
@@ -231,11 +235,13 @@ __global__ void __launch_bounds__(32 * (WARPS + 3), 16 / WARPS)
     const uint32_t tmem = tmem_slot;
     const int n16 = (tile.rows + 15) & ~15;
     const uint32_t idesc = idesc_bf16(C::kF, n16, MODE == MODE_FWD ? 0 : 1, 0);
-    // weights: FWD K-major (64-wide chunks of 16 KiB, 32 bytes per K step), DX MN-major (two
-    // 64-feature atoms of BK contraction rows, 16 rows = 2 KiB per K step); activations
-    // K-major in 64-wide chunks
+    // weights: FWD K-major (64-wide chunks of FEAT rows, 32 bytes per K step), DX MN-major
+    // (64-feature atoms of BK contraction rows, 16 rows = 2 KiB per K step); activations
+    // K-major in 64-wide chunks. Rows 64-127 of a 64-feature tile are what follows in the
+    // shared memory: at most 16 KiB past the weights, less than the code ring behind the
+    // last stage.
     const uint32_t base = smem_u32(smem);
-    const uint64_t ad0 = MODE == MODE_FWD ? smem_desc_sw128(base, 16, 1024) : smem_desc_sw128(base, kA / 2, 1024);
+    const uint64_t ad0 = MODE == MODE_FWD ? smem_desc_sw128(base, 16, 1024) : smem_desc_sw128(base, BK * 128, 1024);
     const uint64_t bd0 = smem_desc_sw128(base + kA, 16, 1024);
     const uint32_t chunk = static_cast<uint32_t>(p.box_rows) * 128 >> 4;  // of the activations, in descriptor units
     const uint32_t step = static_cast<uint32_t>(p.stage_bytes) >> 4;
@@ -248,7 +254,7 @@ __global__ void __launch_bounds__(32 * (WARPS + 3), 16 / WARPS)
       const uint64_t ad = ad0 + so, bd = bd0 + so;
 #pragma unroll
       for (int kk = 0; kk < BK / 16; ++kk)
-        umma_bf16_elect(tmem, ad + ((MODE == MODE_FWD ? (kk >> 2) * 16384 + (kk & 3) * 32 : kk * 2048) >> 4),
+        umma_bf16_elect(tmem, ad + ((MODE == MODE_FWD ? (kk >> 2) * (FEAT * 128) + (kk & 3) * 32 : kk * 2048) >> 4),
                         bd + (kk >> 2) * chunk + ((kk & 3) * 32 >> 4), idesc, (it > 0 || kk > 0) ? 1u : 0u);
       umma_commit_elect(&empty[s]);
       so += step;
@@ -265,10 +271,10 @@ __global__ void __launch_bounds__(32 * (WARPS + 3), 16 / WARPS)
     // The warps form GROUPS groups; group g decodes stages g, g + GROUPS, ..., kUnits
     // 32-weight units per thread and stage, so one proxy fence and one barrier arrival
     // serve kUnits units and GROUPS stages are being decoded at a time. FWD: a stage is
-    // 128 feature rows x BK k; DX: BK contraction rows x 128 feature columns. The 8 lanes
+    // FEAT feature rows x BK k; DX: BK contraction rows x FEAT feature columns. The 8 lanes
     // that share a shared-memory wavefront hold 8 different rows.
     constexpr int kGroupThreads = 32 * WARPS / GROUPS;
-    constexpr int kAcross = MODE == MODE_FWD ? BK / 32 : 4;   // units of a row
+    constexpr int kAcross = MODE == MODE_FWD ? BK / 32 : FEAT / 32;  // units of a row
     constexpr int kRowStep = kGroupThreads / kAcross;         // rows between a thread's units
     const int grp = threadIdx.x / kGroupThreads;
     const int u = threadIdx.x % kGroupThreads;
@@ -320,7 +326,7 @@ __global__ void __launch_bounds__(32 * (WARPS + 3), 16 / WARPS)
     uint32_t off[4];
 #pragma unroll
     for (int c = 0; c < 4; ++c)
-      off[c] = (q >> 1) * (MODE == MODE_FWD ? 16384 : kA / 2) + row * 128 + (((4 * (q & 1) + c) ^ (row & 7)) << 4);
+      off[c] = (q >> 1) * (MODE == MODE_FWD ? FEAT * 128 : BK * 128) + row * 128 + (((4 * (q & 1) + c) ^ (row & 7)) << 4);
     __syncwarp();
     start();
     bool ok = true;
@@ -393,7 +399,7 @@ __global__ void __launch_bounds__(32 * (WARPS + 3), 16 / WARPS)
     const uint32_t t_row = tmem_slot + (static_cast<uint32_t>((warp & 3) * 32) << 16);
     const uint32_t tokens_smem = smem_u32(smem);
 #pragma unroll 1
-    for (int c = 32 * (warp >> 2); c < tile.rows; c += 8 * WARPS) {
+    for (int c = 32 * (warp >> 2); c < tile.rows && (warp & 3) < FEAT / 32; c += 8 * WARPS) {
       uint32_t v[32];
       tmem_ld32(t_row + c, v);
       tmem_ld_wait();
@@ -407,7 +413,7 @@ __global__ void __launch_bounds__(32 * (WARPS + 3), 16 / WARPS)
     asm volatile("barrier.sync 2, %0;" ::"n"(32 * WARPS) : "memory");
     uint16_t *out = p.out + static_cast<int64_t>(tile.row0) * F + f0;
     const int f = 8 * (threadIdx.x & 15);
-    if (f0 + f < F) {
+    if (f < FEAT && f0 + f < F) {
       for (int t = threadIdx.x >> 4; t < tile.rows; t += 2 * WARPS) {
         const uint4 v = lds128(tokens_smem + (t * C::kF + f) * 2);
         *reinterpret_cast<uint4 *>(out + static_cast<int64_t>(t) * F + f) = v;
@@ -423,12 +429,12 @@ __global__ void __launch_bounds__(32 * (WARPS + 3), 16 / WARPS)
   }
 }
 
-template <int MODE, int FMT, int BK, int WARPS, int GROUPS>
+template <int MODE, int FMT, int BK, int WARPS, int GROUPS, int FEAT>
 cudaError_t launch_one(const FewParams &p, const FewMaps &maps, int64_t units, int smem, cudaStream_t stream) {
   static int done_mask = 0;  // per device ordinal (first 31)
   int dev = 0;
   cudaGetDevice(&dev);
-  const auto kernel = sq_gemm_few_kernel<MODE, FMT, BK, WARPS, GROUPS>;
+  const auto kernel = sq_gemm_few_kernel<MODE, FMT, BK, WARPS, GROUPS, FEAT>;
   if (!(done_mask & (1 << (dev & 31)))) {
     cudaError_t e;
     if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -442,13 +448,13 @@ cudaError_t launch_one(const FewParams &p, const FewMaps &maps, int64_t units, i
   return cudaGetLastError();
 }
 
-template <int BK, int WARPS, int GROUPS>
+template <int BK, int WARPS, int GROUPS, int FEAT>
 cudaError_t launch_shape(const FewArgs &a, const FewParams &p, const FewMaps &maps, int smem, cudaStream_t stream) {
   if (a.mode == MODE_FWD)
-    return a.fmt == 0 ? launch_one<MODE_FWD, 0, BK, WARPS, GROUPS>(p, maps, a.units, smem, stream)
-                      : launch_one<MODE_FWD, 1, BK, WARPS, GROUPS>(p, maps, a.units, smem, stream);
-  return a.fmt == 0 ? launch_one<MODE_DX, 0, BK, WARPS, GROUPS>(p, maps, a.units, smem, stream)
-                    : launch_one<MODE_DX, 1, BK, WARPS, GROUPS>(p, maps, a.units, smem, stream);
+    return a.fmt == 0 ? launch_one<MODE_FWD, 0, BK, WARPS, GROUPS, FEAT>(p, maps, a.units, smem, stream)
+                      : launch_one<MODE_FWD, 1, BK, WARPS, GROUPS, FEAT>(p, maps, a.units, smem, stream);
+  return a.fmt == 0 ? launch_one<MODE_DX, 0, BK, WARPS, GROUPS, FEAT>(p, maps, a.units, smem, stream)
+                    : launch_one<MODE_DX, 1, BK, WARPS, GROUPS, FEAT>(p, maps, a.units, smem, stream);
 }
 
 }  // namespace
@@ -456,7 +462,7 @@ cudaError_t launch_shape(const FewArgs &a, const FewParams &p, const FewMaps &ma
 cudaError_t launch_few(const FewArgs &a, const CUtensorMap (&tmX)[3], const CUtensorMap &tmCodes, int sm_count,
                        cudaStream_t stream) {
   const FewMaps maps = {{tmX[0], tmX[1], tmX[2]}, tmCodes};
-  const FewRing ring = few_ring(a.tile_tokens, a.units <= sm_count);
+  const FewRing ring = few_ring(a.tile_tokens, a.units <= sm_count, a.features);
   if (ring.slots < 2) return cudaErrorInvalidValue;
   FewParams p;
   p.scales = a.scales;
@@ -468,15 +474,18 @@ cudaError_t launch_few(const FewArgs &a, const CUtensorMap (&tmX)[3], const CUte
   p.err = a.err;
   p.tiles = a.tiles;
   p.tile_tokens = a.tile_tokens;
-  p.ftiles = static_cast<int>(((a.mode == MODE_FWD ? a.N : a.K) + kFewFeatures - 1) / kFewFeatures);
+  p.ftiles = static_cast<int>(((a.mode == MODE_FWD ? a.N : a.K) + a.features - 1) / a.features);
   p.box_rows = few_box_rows(a.tile_tokens);
   p.stage_bytes = ring.stage_bytes;
   p.stages = ring.stages;
   p.slots = ring.slots;
   for (p.tmem_cols = 32; p.tmem_cols < a.tile_tokens; p.tmem_cols *= 2) {
   }
-  return ring.depth == 128 ? launch_shape<128, 16, kFewGroups>(a, p, maps, ring.bytes, stream)
-                           : launch_shape<64, 8, kFewGroups>(a, p, maps, ring.bytes, stream);
+  if (a.features == kFewNarrow)
+    return ring.depth == 128 ? launch_shape<128, 16, kFewGroupsNarrow, kFewNarrow>(a, p, maps, ring.bytes, stream)
+                             : cudaErrorInvalidValue;
+  return ring.depth == 128 ? launch_shape<128, 16, kFewGroups, kFewFeatures>(a, p, maps, ring.bytes, stream)
+                           : launch_shape<64, 8, kFewGroups, kFewFeatures>(a, p, maps, ring.bytes, stream);
 }
 
 }  // namespace sqi

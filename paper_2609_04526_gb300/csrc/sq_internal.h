@@ -100,8 +100,11 @@ constexpr int kFewBoxRows = 32;        // tokens of the smallest TMA box
 constexpr int kFewSmemBytes = 111 * 1024;  // of a CTA: two share an SM
 constexpr int kFewSmemAlone = 224 * 1024;  // ... where the launch has at most one CTA per SM
 constexpr int kFewSlotBytes = 128 * 64;    // packed codes of 128 x 128 weights
-constexpr int kFewMaxStages = 3, kFewMaxSlots = 12;
-constexpr int kFewGroups = 2;              // sets of decode warps, which take the stages in turn
+constexpr int kFewMaxStages = 4, kFewMaxSlots = 12;
+constexpr int kFewGroups = 2;        // sets of decode warps, which take the stages in turn
+constexpr int kFewGroupsNarrow = 4;  // ... of tiles of kFewNarrow features
+constexpr int kFewNarrow = 64;       // features of a tile where twice the tiles still have an SM each
+constexpr int kFewTokensNarrow = 96; // ... and few enough tokens for four stages
 
 // Tokens of the equal tiles (whole MMA steps of 16) that `rows` tokens are cut into.
 inline int few_tile_tokens(int64_t rows, int limit) {
@@ -121,26 +124,28 @@ inline int few_box_rows(int tile_tokens) {
 // slot of its next stage. That wait can only be told from one for an earlier use of the slot
 // if the use before is known to have landed: because the same set read it (a slot's uses lie
 // slots * 128 / depth stages apart), or because its MMAs are done (a set that starts on stage
-// i has seen those of stage i - kFewGroups - stages). A slot count that gives neither loses
-// one. (Four stages, three slots and four sets for up to 32 tokens gave neither.)
+// i has seen those of stage i - sets - stages). A slot count that gives neither is reduced.
+// (Four stages, three slots and four sets for up to 32 tokens gave neither.)
 struct FewRing {
   int depth, stage_bytes, stages, slots;
   int bytes;  // with 1 KiB for the alignment
 };
-inline FewRing few_ring(int tile_tokens, bool alone) {
+inline FewRing few_ring(int tile_tokens, bool alone, int features = kFewFeatures) {
   FewRing r;
   const int rows = few_box_rows(tile_tokens);
   const int room = (alone ? kFewSmemAlone : kFewSmemBytes) - 1024;
   r.depth = alone ? 128 : 64;
-  r.stage_bytes = (kFewFeatures + rows) * r.depth * 2;
-  if (alone)
+  r.stage_bytes = (features + rows) * r.depth * 2;
+  if (features == kFewNarrow)
+    r.stages = 4;
+  else if (alone)
     r.stages = rows <= 96 ? 3 : 2;
   else
     r.stages = rows <= 64 ? 3 : 2;
   r.slots = (room - r.stages * r.stage_bytes) / kFewSlotBytes;
   if (r.slots > kFewMaxSlots) r.slots = kFewMaxSlots;
-  const int reuse = r.slots * (128 / r.depth);
-  if (reuse % kFewGroups != 0 && reuse < kFewGroups + r.stages) --r.slots;
+  const int sets = features == kFewNarrow ? kFewGroupsNarrow : kFewGroups, per = 128 / r.depth;
+  while (r.slots * per % sets != 0 && r.slots * per < sets + r.stages) --r.slots;
   r.bytes = r.stages * r.stage_bytes + r.slots * kFewSlotBytes + 1024;
   return r;
 }
@@ -149,6 +154,15 @@ struct FewTile {
   int expert, row0, rows;
   float ws2;
 };
+// Features of a tile. A CTA that decodes half as many weights per stage, in four sets of
+// warps with a stage each, takes 0.43 us for one where 128 features take 0.56, so tiles of 64
+// where twice as many still have an SM of their own (4096 x 4096 at 187 tokens 22.6 -> 18.5
+// us); with more tokens than four stages have room for they were no faster.
+inline int few_features(int64_t token_tiles, int tile_tokens, int64_t features, int sm_count) {
+  return tile_tokens <= kFewTokensNarrow && token_tiles * ((features + kFewNarrow - 1) / kFewNarrow) <= sm_count
+             ? kFewNarrow
+             : kFewFeatures;
+}
 struct FewArgs {
   int mode, fmt;
   int64_t M, N, K;
@@ -158,22 +172,25 @@ struct FewArgs {
   int *err;
   const FewTile *tiles;  // device list of a grouped call, or null: tiles of tile_tokens over M
   int tile_tokens;       // tokens of the largest tile (<= kFewTokens)
+  int features;          // output features of a tile (few_features)
   int64_t units;
 };
 // Which kernel runs a forward or input gradient, by estimates of both in microseconds that
 // were fitted to measured launches (weights of 4096 x 4096, 1024 x 4096, 14336 x 4096, 768 x
 // 2048 and 256 x 512 at 16 to 4096 tokens; 128 experts of 768 x 2048 and 2880 x 2880 with 2 to
 // 1024 rows each) and lie within 20 % of them above 15 us. Both sides of the line, few-token
-// against pair kernel, in us: 4096 x 4096 23 against 43 at 16 to 192 tokens, 31 against 45 at
+// against pair kernel, in us: 4096 x 4096 19 against 43 at 16 to 192 tokens, 31 against 45 at
 // 1024, 78 against 45 at 2048; 1024 x 4096 25 against 44 at 2048; 768 x 2048 experts 77 against
 // 127 with 64 rows each, 139 against 148 with 256, 223 against 198 with 512; 2880 x 2880
 // experts 271 against 566 with 16 rows each, 345 against 520 with 128, 581 against 567 with 256.
 //
 // few_us, for token tiles of `tokens` tokens on average: a CTA alone on its SM takes 0.56 us
-// per 128-deep stage, more above 128 tokens (two stages in flight); CTAs that share an SM 0.27
+// per 128-deep stage (of 64 features 0.43), more above 128 tokens (two stages in flight); CTAs that share an SM 0.27
 // us and up with the tokens per 64-deep stage, and 1.5 us to start and drain.
 inline double few_us(int64_t token_tiles, double tokens, int64_t features, int64_t contraction, int sm_count) {
   const int64_t ctas = token_tiles * ((features + kFewFeatures - 1) / kFewFeatures);
+  if (tokens <= kFewTokensNarrow && token_tiles * ((features + kFewNarrow - 1) / kFewNarrow) <= sm_count)
+    return 4.8 + ((contraction + 127) / 128) * 0.43;
   if (ctas <= sm_count)
     return 4.8 + ((contraction + 127) / 128) * (0.56 + (tokens > 128 ? 0.0015 * (tokens - 128) : 0.0));
   const double per_sm = ctas > 4 * sm_count ? static_cast<double>(ctas) / sm_count

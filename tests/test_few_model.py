@@ -25,16 +25,17 @@ int main() {
     auto tiles_at = [&](int limit) { const int t = sqi::few_tile_tokens(M, limit); return (int64_t)((M + t - 1) / t); };
     const int64_t pair = ((M + 511) / 512) * ((F + 255) / 256);
     const int limit = sqi::few_limit(tiles_at, M, F, K, pair, SMS);
-    int tokens = 0, alone = 0;
+    int tokens = 0, alone = 0, feat = 0;
     sqi::FewRing r{};
     double few = 0;
     if (limit) {
       tokens = sqi::few_tile_tokens(M, limit);
       alone = tiles_at(limit) * ((F + 127) / 128) <= SMS;
-      r = sqi::few_ring(tokens, alone);
+      feat = sqi::few_features(tiles_at(limit), tokens, F, SMS);
+      r = sqi::few_ring(tokens, alone, feat);
       few = sqi::few_us(tiles_at(limit), (double)M / tiles_at(limit), F, K, SMS);
     }
-    std::printf("%d %d %d %d %d %d %d %d %.9g %.9g\n", limit, tokens, alone, r.depth, r.stage_bytes, r.stages,
+    std::printf("%d %d %d %d %d %d %d %d %d %.9g %.9g\n", limit, tokens, alone, feat, r.depth, r.stage_bytes, r.stages,
                 r.slots, r.bytes, few, sqi::pair_us(pair, K, SMS));
   }
   return 0;
@@ -65,23 +66,25 @@ def test_every_plan_fits(plan):
     cases = [(log(1 << 31) if i % 4 else log(2000), 8 * log(1 << 21), 32 * log(1 << 19)) for i in range(4000)]
     cases += [(m, f, 4096) for m in range(1, 1100, 7) for f in (8, 128, 136, 1024, 4096, 14336)]
     chosen = 0
-    for (M, F, K), (limit, tokens, alone, depth, stage, stages, slots, nbytes, few, pair) in zip(cases, plan(cases)):
+    for (M, F, K), (limit, tokens, alone, feat, depth, stage, stages, slots, nbytes, few, pair) in zip(cases, plan(cases)):
         if not limit:
             continue
         chosen += 1
         assert few < 0.97 * pair
         assert tokens % 16 == 0 and 16 <= tokens <= limit <= 256 and (tokens <= 192 or alone)
-        assert depth == (128 if alone else 64) and stage == (128 + math.ceil(tokens / 32) * 32) * depth * 2
-        assert 2 <= stages <= 3 and 2 <= slots <= 12
+        assert depth == (128 if alone else 64) and stage == (feat + math.ceil(tokens / 32) * 32) * depth * 2
+        assert (stages == 4 if feat == 64 else 2 <= stages <= 3) and 2 <= slots <= 12
         assert nbytes == stages * stage + slots * 8192 + 1024
         # shared memory of a CTA (227 KiB less the static part), or of two on an SM (228 KiB less 1 KiB each)
         assert nbytes + 512 <= 227 * 1024 if alone else 2 * (nbytes + 512 + 1024) <= 228 * 1024
         assert tokens * 256 <= nbytes - 1024  # the epilogue's bf16 tile
-        # a set of decode warps (of two) can tell its use of a code slot from the use before
-        reuse = slots * 128 / depth
-        assert reuse % 2 == 0 or reuse >= 2 + stages
+        # a set of decode warps can tell its use of a code slot from the use before
+        reuse, sets = slots * 128 / depth, 4 if feat == 64 else 2
+        assert (reuse % sets == 0 or reuse >= sets + stages) and sets <= max(stages, 2)
+        if feat == 64:  # the MMAs' rows past the tile's read no further than the code ring
+            assert alone and tokens <= 96 and slots * 8192 > 16384
         # the codes run ahead of the stages in flight
-        assert slots >= math.ceil(stages * depth / 128) + (0 if depth == 128 and stages == 2 else 1)
+        assert slots >= math.ceil(stages * depth / 128) + (0 if depth == 128 and stages in (2, 4) else 1)
     assert chosen > 500
 
 

@@ -149,3 +149,22 @@ def test_few_token_and_pair_kernels_agree_bit_for_bit():
         Yf, dXf = h.sq_fwd(w, X[:100]), h.sq_bwd_dx(w, dY[:100])
         h.sq_sync()
         assert torch.equal(Y[:100], Yf) and torch.equal(dX[:100], dXf)
+
+
+@pytest.mark.parametrize("fmt", [0, 1])
+@pytest.mark.parametrize("M,N,K", [(1, 72, 4128), (96, 4104, 1056), (33, 2056, 544), (190, 4128, 288), (16, 9728, 96)])
+def test_few_token_tiles_of_64_features(fmt, M, N, K):
+    """Tiles of 64 features: ragged last tiles, one to three 32-token boxes, two token tiles,
+    contractions shorter and longer than the code ring; each row as in a large batch, bit for bit."""
+    import paper_2609_04526_gb300 as pkg
+    from paper_2609_04526_gb300 import synth
+    h = pkg.Handle()
+    wl = synth.custom("few", fmt, 4096, N, K, seed=M + N + K, kind="outlier")
+    w, X, dY = setup_linear(wl, wl.linears[0])
+    Y, dX = h.sq_fwd(w, X[:M]), h.sq_bwd_dx(w, dY[:M])
+    Yb, dXb = h.sq_fwd(w, X), h.sq_bwd_dx(w, dY)
+    h.sq_sync()
+    codes, scales = host(w.codes), host(w.scales)
+    assert_close(f64(Y), oracle.fwd(fmt, codes, scales, w.ws2, hbits(X[:M])), what="Y")
+    assert_close(f64(dX), oracle.dx(fmt, codes, scales, w.ws2, hbits(dY[:M])), what="dX")
+    assert torch.equal(Y, Yb[:M]) and torch.equal(dX, dXb[:M])
