@@ -631,6 +631,7 @@ __global__ void __launch_bounds__(kThreads) sq_swap_or_diff_kernel(int64_t count
 // results do not change between runs.
 constexpr int kT = 64;   // output tile edge
 constexpr int kTP = 68;  // padded row of a staged operand (16-byte multiple; spreads the transposed stores)
+constexpr int lowrank_smem(int r) { return (kTP + kT) * r * static_cast<int>(sizeof(float)); }  // <= 132 KiB
 
 __device__ __forceinline__ float bf16_bits(uint16_t h) { return __uint_as_float(static_cast<uint32_t>(h) << 16); }
 
@@ -1314,6 +1315,19 @@ cudaError_t launch_merge_planes(int fmt, const PlaneTable &t, int64_t *acc, cuda
   return cudaGetLastError();
 }
 
+// Opens the kernel's limit of dynamic shared memory on the current device, once and to the
+// largest size that it is ever launched with: the limit belongs to the device, so a call that
+// set it to its own size could refuse the launch of another thread's larger one.
+template <class Kernel>
+static cudaError_t allow_smem(Kernel kernel, int most, int *done_mask) {
+  int dev = 0;
+  cudaGetDevice(&dev);
+  if (*done_mask & (1 << (dev & 31))) return cudaSuccess;
+  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  if (e == cudaSuccess) *done_mask |= 1 << (dev & 31);  // per device ordinal (first 31)
+  return e;
+}
+
 template <int FMT>
 static cudaError_t launch_wide(int64_t N, int64_t G, int r, float ws2, float cap, const float *ws2_per,
                                float alpha_over_r, const uint8_t *base, const uint16_t *B, const uint16_t *A,
@@ -1321,13 +1335,26 @@ static cudaError_t launch_wide(int64_t N, int64_t G, int r, float ws2, float cap
                                cudaStream_t stream, int experts) {
   const dim3 grid(static_cast<unsigned>((N + kWideRows - 1) / kWideRows),
                   static_cast<unsigned>((G + kWideCols - 1) / kWideCols), static_cast<unsigned>(experts));
-  const int smem = wide_smem(r);  // <= 50 KiB
-  const cudaError_t e = cudaFuncSetAttribute(sq_project_lowrank_wide_kernel<FMT>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  static int done_mask = 0;
+  const cudaError_t e = allow_smem(sq_project_lowrank_wide_kernel<FMT>, wide_smem(kWideChunk), &done_mask);
   if (e != cudaSuccess) return e;
-  sq_project_lowrank_wide_kernel<FMT><<<grid, kWideThreads, smem, stream>>>(N, G, r, ws2, cap, ws2_per, alpha_over_r,
-                                                                            base, B, A, bytes_out, mask_out, nonfinite,
-                                                                            latent_out);
+  sq_project_lowrank_wide_kernel<FMT><<<grid, kWideThreads, wide_smem(r), stream>>>(
+      N, G, r, ws2, cap, ws2_per, alpha_over_r, base, B, A, bytes_out, mask_out, nonfinite, latent_out);
+  return cudaGetLastError();
+}
+
+template <int FMT>
+static cudaError_t launch_lowrank(int64_t N, int64_t G, int r, float ws2, float cap, const float *ws2_per,
+                                  float alpha_over_r, const uint8_t *base, const uint16_t *B, const uint16_t *A,
+                                  uint8_t *bytes_out, uint8_t *mask_out, int32_t *nonfinite, float *latent_out,
+                                  cudaStream_t stream, int experts) {
+  const dim3 grid(static_cast<unsigned>((N + kT - 1) / kT), static_cast<unsigned>((G + kT - 1) / kT),
+                  static_cast<unsigned>(experts));
+  static int done_mask = 0;
+  const cudaError_t e = allow_smem(sq_project_lowrank_kernel<FMT>, lowrank_smem(kMaxLowRank), &done_mask);
+  if (e != cudaSuccess) return e;
+  sq_project_lowrank_kernel<FMT><<<grid, kThreads, lowrank_smem(r), stream>>>(
+      N, G, r, ws2, cap, ws2_per, alpha_over_r, base, B, A, bytes_out, mask_out, nonfinite, latent_out);
   return cudaGetLastError();
 }
 
@@ -1349,24 +1376,10 @@ cudaError_t launch_project_lowrank(int fmt, int64_t N, int64_t G, int r, float w
                                      nonfinite, latent_out, stream, experts)
                     : launch_wide<1>(N, G, r, ws2, cap, nullptr, alpha_over_r, base, B, A, bytes_out, mask_out,
                                      nonfinite, latent_out, stream, experts);
-  const dim3 grid(static_cast<unsigned>((N + kT - 1) / kT), static_cast<unsigned>((G + kT - 1) / kT),
-                  static_cast<unsigned>(experts));
-  const size_t smem = static_cast<size_t>(kTP + kT) * r * sizeof(float);  // <= 132 KiB for r <= 256
-  cudaError_t e;
-  if (fmt == 0) {
-    if ((e = cudaFuncSetAttribute(sq_project_lowrank_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  static_cast<int>(smem))) != cudaSuccess)
-      return e;
-    sq_project_lowrank_kernel<0><<<grid, kThreads, smem, stream>>>(N, G, r, ws2, cap, ws2_per, alpha_over_r, base,
-                                                                   B, A, bytes_out, mask_out, nonfinite, latent_out);
-  } else {
-    if ((e = cudaFuncSetAttribute(sq_project_lowrank_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  static_cast<int>(smem))) != cudaSuccess)
-      return e;
-    sq_project_lowrank_kernel<1><<<grid, kThreads, smem, stream>>>(N, G, r, ws2, cap, nullptr, alpha_over_r, base,
-                                                                   B, A, bytes_out, mask_out, nonfinite, latent_out);
-  }
-  return cudaGetLastError();
+  return fmt == 0 ? launch_lowrank<0>(N, G, r, ws2, cap, ws2_per, alpha_over_r, base, B, A, bytes_out, mask_out,
+                                      nonfinite, latent_out, stream, experts)
+                  : launch_lowrank<1>(N, G, r, ws2, cap, nullptr, alpha_over_r, base, B, A, bytes_out, mask_out,
+                                      nonfinite, latent_out, stream, experts);
 }
 
 // Workspace of the adapter gradients: the partial products of dB and of dA (all experts).
