@@ -289,11 +289,11 @@ __global__ void __launch_bounds__(kAtThreads, 2)
       umma_commit_elect(bar);
     }
     if (s + 1 < steps) load(s + 1);  // in flight during the MMAs
-    if (!(ok = mbar_wait(bar, static_cast<uint32_t>(s) & 1u, abort_flag, err))) break;
-    tc_fence_after();
-    // drain this step's dA: lanes j = 32 (warp % 4) + lane, columns b 32 (warp / 4) .. + 31
-    const int j = (warp & 3) * 32 + lane;
-    {
+    ok = mbar_wait(bar, static_cast<uint32_t>(s) & 1u, abort_flag, err);
+    if (__all_sync(0xFFFFFFFFu, ok)) {
+      tc_fence_after();
+      // drain this step's dA: lanes j = 32 (warp % 4) + lane, columns b 32 (warp / 4) .. + 31
+      const int j = (warp & 3) * 32 + lane;
       const int c0 = 32 * col_half;
       uint32_t v[32];
       tmem_ld32(tmem + t_lane + 128 + (s & 1) * kAtStep + c0, v);
@@ -311,7 +311,10 @@ __global__ void __launch_bounds__(kAtThreads, 2)
       }
     }
     tc_fence_before();
-    __syncthreads();  // shared memory and this dA buffer are free for the next step
+    // Shared memory and this dA buffer are free for the next step. If the wait ran out for some
+    // threads only, all leave here together: none is missing at a later barrier or election.
+    ok = __syncthreads_and(ok);
+    if (!ok) break;
   }
   if (ok && dB_all && steps > 0) {
     tc_fence_after();

@@ -1,0 +1,22 @@
+"""How kernels end after a wait that ran out (checked on the source: nothing makes a wait of these
+kernels run out on a GPU)."""
+import os
+import re
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2609_04526_gb300", "csrc")
+
+
+def _source(name):
+    with open(os.path.join(CSRC, name)) as f:
+        return re.sub(r"//[^\n]*", "", f.read())
+
+
+def test_adapter_gradient_gives_up_as_a_block():
+    """A bounded wait can run out for some of a block's threads only. The adapter gradient's steps
+    have block barriers and elections of whole warps, which wait without a limit for threads that
+    left: its loop may end on the block's vote alone."""
+    src = _source("sq_adapter_tc.cu")
+    loop = src[src.index("for (int s = 0; s < steps; ++s)"):src.index("if (ok && dB_all")]
+    exits = re.findall(r"if \(([^;{}]*)\) (?:break|return);", loop)
+    assert exits == ["!ok"], exits
+    assert re.search(r"ok = __syncthreads_and\(ok\);\s*if \(!ok\) break;", loop)
