@@ -344,9 +344,10 @@ __global__ void __launch_bounds__(kAtThreads, 2)
       for (int64_t i = threadIdx.x; i < count; i += kAtThreads) dst[i] = tile[i];
     }
   }
-  if (!ok && threadIdx.x == 0) {  // a wait ran out: let this CTA's MMAs finish before TMEM is freed
-    umma_commit(bar + 3);
+  if (!ok && warp == 0) {  // a wait ran out: let this CTA's MMAs finish before TMEM is freed
+    umma_commit_elect(bar + 3);  // a commit waits for its own lane's MMAs: the lane that issued them
     mbar_drain(bar + 3, 0);
+    __syncwarp();
   }
   tc_fence_before();
   __syncthreads();

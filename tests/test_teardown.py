@@ -3,6 +3,8 @@ kernels run out on a GPU)."""
 import os
 import re
 
+import pytest
+
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2609_04526_gb300", "csrc")
 
 
@@ -20,3 +22,13 @@ def test_adapter_gradient_gives_up_as_a_block():
     exits = re.findall(r"if \(([^;{}]*)\) (?:break|return);", loop)
     assert exits == ["!ok"], exits
     assert re.search(r"ok = __syncthreads_and\(ok\);\s*if \(!ok\) break;", loop)
+
+
+@pytest.mark.parametrize("name", sorted(n for n in os.listdir(CSRC) if n.endswith((".cu", ".cuh"))))
+def test_commits_come_from_the_lane_that_issued(name):
+    """tcgen05.commit waits for the MMAs of the thread that executes it. Where an elected lane
+    issues them, a commit by a fixed thread (before TMEM is freed, say) need not wait for any."""
+    src = _source(name)
+    if "umma_bf16_elect(" in src:
+        assert not re.findall(r"\bumma_commit\(", src)
+        assert "umma_commit_elect(" in src
