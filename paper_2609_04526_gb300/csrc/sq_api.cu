@@ -536,12 +536,16 @@ sq_status run_grouped(sq_handle h, int mode, const sq_grouped_weight *w, const s
         }
       return tiles;
     };
-    const int limit = sqi::few_limit(tiles_at, offsets[E], F, Kc, total, dev->sm_count);
-    if (limit > 0) {
-      const int64_t token_tiles = tiles_at(limit);
-      int tokens = 0;  // of the largest token tile
+    auto largest_at = [&](int limit) {
+      int tokens = 0;
       for (int x = 0; x < E; ++x)
         if (rows[x] > 0) tokens = std::max(tokens, sqi::few_tile_tokens(rows[x], limit));
+      return tokens;
+    };
+    const int limit = sqi::few_limit(tiles_at, offsets[E], F, Kc, total, dev->sm_count, largest_at);
+    if (limit > 0) {
+      const int64_t token_tiles = tiles_at(limit);
+      const int tokens = largest_at(limit);
       TableSlot *t = nullptr;
       const size_t bytes = static_cast<size_t>(token_tiles) * sizeof(sqi::FewTile);
       SQ_TRY(acquire_table(h, dev, bytes, &t));

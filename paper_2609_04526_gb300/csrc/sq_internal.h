@@ -178,21 +178,26 @@ struct FewArgs {
 // Which kernel runs a forward or input gradient, by estimates of both in microseconds that
 // were fitted to measured launches (weights of 4096 x 4096, 1024 x 4096, 14336 x 4096, 768 x
 // 2048 and 256 x 512 at 16 to 4096 tokens; 128 experts of 768 x 2048 and 2880 x 2880 with 2 to
-// 1024 rows each) and lie within 20 % of them above 15 us. Both sides of the line, few-token
+// 1024 rows each). Over 346 launches of these and a few more shapes that ran on both kernels,
+// the estimates above 15 us lie within 30 % of the times (half of them within 10 %), and the
+// choice was the faster kernel or at most 7 % slower than it. Both sides of the line, few-token
 // against pair kernel, in us: 4096 x 4096 19 against 43 at 16 to 192 tokens, 31 against 45 at
 // 1024, 78 against 45 at 2048; 1024 x 4096 25 against 44 at 2048; 768 x 2048 experts 77 against
 // 127 with 64 rows each, 139 against 148 with 256, 223 against 198 with 512; 2880 x 2880
 // experts 271 against 566 with 16 rows each, 345 against 520 with 128, 581 against 567 with 256.
 //
-// few_us, for token tiles of `tokens` tokens on average: a CTA alone on its SM takes 0.56 us
-// per 128-deep stage (of 64 features 0.43), more above 128 tokens (two stages in flight); CTAs that share an SM 0.27
-// us and up with the tokens per 64-deep stage, and 1.5 us to start and drain.
-inline double few_us(int64_t token_tiles, double tokens, int64_t features, int64_t contraction, int sm_count) {
+// few_us, for token tiles of `tokens` tokens on average and `largest` at most (0: all alike): a
+// CTA alone on its SM takes 0.56 us per 128-deep stage (of 64 features 0.43), more above 128
+// tokens (two stages in flight), and the launch lasts as long as its largest tile; CTAs that
+// share an SM 0.27 us and up with the tokens per 64-deep stage, and 1.5 us to start and drain.
+inline double few_us(int64_t token_tiles, double tokens, int64_t features, int64_t contraction, int sm_count,
+                     int largest = 0) {
   const int64_t ctas = token_tiles * ((features + kFewFeatures - 1) / kFewFeatures);
-  if (tokens <= kFewTokensNarrow && token_tiles * ((features + kFewNarrow - 1) / kFewNarrow) <= sm_count)
+  const double most = largest > 0 ? largest : tokens;
+  if (most <= kFewTokensNarrow && token_tiles * ((features + kFewNarrow - 1) / kFewNarrow) <= sm_count)
     return 4.8 + ((contraction + 127) / 128) * 0.43;
   if (ctas <= sm_count)
-    return 4.8 + ((contraction + 127) / 128) * (0.56 + (tokens > 128 ? 0.0015 * (tokens - 128) : 0.0));
+    return 4.8 + ((contraction + 127) / 128) * (0.56 + (most > 128 ? 0.0015 * (most - 128) : 0.0));
   const double per_sm = ctas > 4 * sm_count ? static_cast<double>(ctas) / sm_count
                                             : static_cast<double>((ctas + sm_count - 1) / sm_count);
   return 4.8 + per_sm * (((contraction + 63) / 64) * (0.27 + 0.0006 * tokens) + 1.5);
@@ -204,10 +209,11 @@ inline double pair_us(int64_t tiles, int64_t contraction, int sm_count) {
 }
 // The limit of a token tile (few_tile_tokens) of the few-token launch over `rows` tokens in
 // all, or 0 where the pair kernel's `pair_tiles` tiles are the faster launch. `tiles_at`
-// counts the token tiles at a limit.
-template <class TilesAt>
+// counts the token tiles at a limit, `largest_at` gives the tokens of the largest of them
+// (where experts differ).
+template <class TilesAt, class LargestAt>
 inline int few_limit(TilesAt tiles_at, int64_t rows, int64_t features, int64_t contraction, int64_t pair_tiles,
-                     int sm_count) {
+                     int sm_count, LargestAt largest_at) {
   if (sm_count < 2) return 0;
   double best_us = 0.97 * pair_us(pair_tiles, contraction, sm_count);
   int best = 0;
@@ -215,13 +221,19 @@ inline int few_limit(TilesAt tiles_at, int64_t rows, int64_t features, int64_t c
     const int64_t tiles = tiles_at(limit);
     const int64_t ctas = tiles * ((features + kFewFeatures - 1) / kFewFeatures);
     if (ctas > (int64_t(1) << 24) || (limit > kFewTokensShared && ctas > sm_count)) continue;
-    const double us = few_us(tiles, static_cast<double>(rows) / tiles, features, contraction, sm_count);
+    const double us =
+        few_us(tiles, static_cast<double>(rows) / tiles, features, contraction, sm_count, largest_at(limit));
     if (us < best_us) {
       best_us = us;
       best = limit;
     }
   }
   return best;
+}
+template <class TilesAt>
+inline int few_limit(TilesAt tiles_at, int64_t rows, int64_t features, int64_t contraction, int64_t pair_tiles,
+                     int sm_count) {
+  return few_limit(tiles_at, rows, features, contraction, pair_tiles, sm_count, [](int) { return 0; });
 }
 
 // tmX: the activations [M, contraction] in boxes of 64 x kFewBoxRows, 2 kFewBoxRows

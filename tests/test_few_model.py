@@ -95,3 +95,17 @@ def test_measured_sides(plan):
              (4096, 4096, 4096): False, (1999, 4096, 14336): False, (32768, 14336, 4096): False}
     for case, r in zip(sides, plan(list(sides))):
         assert bool(r[0]) == sides[case], case
+
+
+@pytest.mark.parametrize("rows,F,K", [([128, 16, 16, 16], 1024, 4096), ([97, 1, 1], 640, 2080), ([8] * 7 + [256], 512, 2048),
+                                      ([96, 5, 60], 1024, 4096), ([192] + [3] * 12, 1024, 1024)])
+def test_estimate_is_of_the_launched_shape(rows, F, K):
+    """Ragged experts: the tile shape follows the largest tile, and so does the estimate."""
+    from few_plan import plan as plan_of
+    p = plan_of(rows, F, K)
+    if p is None:
+        pytest.skip("no host C++ compiler or CUDA headers")
+    assert p.limit and p.ctas <= SMS
+    stage = 0.43 if p.features == 64 else 0.56 + 0.0015 * max(0, p.largest - 128)
+    assert p.features == (64 if p.largest <= 96 and p.tiles * math.ceil(F / 64) <= SMS else 128)
+    assert math.isclose(p.few_us, 4.8 + math.ceil(K / 128) * stage, rel_tol=1e-6)
