@@ -218,9 +218,11 @@ __global__ void __launch_bounds__(32 * (WARPS + 3), 16 / WARPS)
         ph ^= 1u;
       }
     }
-    // after an abort: wait, with a limit, for the copies in flight (an aborted stage may
-    // never complete its other arrivals, so only for the last of those)
-    if (*abort_flag && it > 0) mbar_drain(&full[(it - 1) % S], static_cast<uint32_t>((it - 1) / S) & 1u);
+    // after an abort: wait, with a limit, for the copies in flight (of every stage: the last
+    // one's may land first; a stage that its decode warps gave up only ends at the limit)
+    if (*abort_flag) {
+      for (int i = (it > S ? it - S : 0); i < it; ++i) mbar_drain(&full[i % S], static_cast<uint32_t>(i / S) & 1u);
+    }
     __syncwarp();
   } else if (warp == kMmaWarp) {
     // ------------------------------------------------------ MMA issuer

@@ -32,3 +32,14 @@ def test_commits_come_from_the_lane_that_issued(name):
     if "umma_bf16_elect(" in src:
         assert not re.findall(r"\bumma_commit\(", src)
         assert "umma_commit_elect(" in src
+
+
+def test_aborted_copies_are_waited_for():
+    """After an abort every copy in flight is waited for, ring by ring: in the few-token kernel the
+    codes (slots) and the activations (stages). A block that ends before a copy lands lets it write
+    into the next block's shared memory."""
+    src = re.sub(r"\s+", " ", _source("sq_few.cu"))
+    for bar, count, filled in (("cfull", "p.slots", "j"), ("full", "S", "it")):
+        loop = (rf"if \(\*abort_flag\) {{ for \(int i = \({filled} > {count} \? {filled} - {count} : 0\); i < {filled}; \+\+i\) "
+                rf"mbar_drain\(&{bar}\[i % {count}\], static_cast<uint32_t>\(i / {count}\) & 1u\);")
+        assert re.search(loop, src), bar
