@@ -1,11 +1,11 @@
 """GPU parity of the grouped expert contractions (Sec. 3 "MoE: a batched
 grouped-expert kernel") against the oracle, through the C ABI.
 
-Small ragged cases (empty experts, experts of 1 row, experts whose rows straddle
-the 512-row tiles, ragged N and K) are compared element by element with the
+Small ragged cases (empty experts, experts of 1 row, several token tiles, ragged N and K; forward and
+input gradient on the few-token kernel) are compared element by element with the
 oracle's grouped definitions; every expert's slice is also bit-identical to the
-dense entry point called on that expert alone (the same kernels, the same
-arithmetic order). The full-size Qwen3-30B-A3B- and gpt-oss-120B-shaped expert
+dense entry point called on that expert alone (the same arithmetic order). Experts at the
+edges of the 512-row tiles beside large ones run on the pair kernel. The full-size Qwen3-30B-A3B- and gpt-oss-120B-shaped expert
 linears are checked on oracle samples of several experts and bit for bit against
 the per-expert dense calls over every output."""
 import numpy as np
@@ -13,6 +13,7 @@ import pytest
 import torch
 
 import oracle
+from few_plan import SMS, plan
 from gpu_util import assert_close, f64, hbits, host
 
 pytestmark = pytest.mark.gpu
@@ -72,7 +73,7 @@ SMALL = [
     ("g_mx_many", MX, [0, 0, 0, 5, 130, 0, 512, 513, 1, 0], 40, 96),
     ("g_nv_tail_empty", NV, [77, 0, 0], 8, 32),
     ("g_nv_long_k", NV, [3, 260], 264, 2080),
-    # 256-row tile halves: exactly one half, one row past it, one short of it, a half past a tile
+    # two to seven token tiles per expert, whole and nearly whole ones
     ("g_nv_half_edges", NV, [256, 257, 255, 768, 769], 264, 512),
 ]
 
@@ -162,7 +163,7 @@ def test_grouped_full_size_sampled(h, key, name):
 def test_table_ring_reuse_with_calls_in_flight(h):
     """More grouped calls than the handle has expert tables, each with its own
     routing and output, enqueued without a sync: every result matches its own
-    per-expert dense calls."""
+    per-expert dense calls (few-token kernel: tables of token tiles)."""
     import paper_2609_04526_gb300 as pkg
     from paper_2609_04526_gb300 import synth
     wl = synth.custom_moe("ring", NV, [1] * 6, 264, 512, seed=5)
@@ -183,6 +184,60 @@ def test_table_ring_reuse_with_calls_in_flight(h):
                                                                            device="cuda"))
         h.sq_sync()
         assert torch.equal(Y, Yd)
+
+
+# beside large experts: none, one row, 256-row halves (one short, exact, one past), a half past a tile
+PAIR_ROWS = [0, 1, 2048, 255, 3072, 256, 257, 2560, 768, 769, 0]
+
+
+def _on_pair_kernel(rows, N, K):
+    assert torch.cuda.get_device_properties(0).multi_processor_count == SMS
+    return plan(rows, N, K).limit == 0 and plan(rows, K, N).limit == 0
+
+
+@pytest.mark.parametrize("fmt", [NV, MX])
+def test_grouped_pair_kernel_edges(h, fmt):
+    """Sizes whose forward and input gradient run on the grouped pair kernel: skipped tile halves,
+    steps over experts without tiles, stores clipped at each expert's rows (stale values behind
+    them belong to the next expert), ragged N and K."""
+    from paper_2609_04526_gb300 import synth
+    N, K = 1032, 1056
+    assert _on_pair_kernel(PAIR_ROWS, N, K)
+    wl = synth.custom_moe("pair", fmt, PAIR_ROWS, N, K, seed=11 + fmt, kind="outlier" if fmt else "gauss")
+    gw, off, X, dY = _setup(wl, wl.linears[0])
+    Y = h.sq_grouped_fwd(gw, off, X, torch.full((off[-1], N), float("nan"), dtype=torch.bfloat16, device="cuda"))
+    dX = h.sq_grouped_bwd_dx(gw, off, dY, torch.full((off[-1], K), float("nan"), dtype=torch.bfloat16, device="cuda"))
+    h.sq_sync()
+    Yd, dXd, _ = _dense_per_expert(h, gw, off, X, dY)
+    h.sq_sync()
+    assert torch.equal(Y, Yd) and torch.equal(dX, dXd)
+    for e, rows in enumerate(PAIR_ROWS):
+        if 0 < rows < 1024:
+            a, b = off[e], off[e + 1]
+            w = gw.expert(e)
+            c, s = host(w.codes), host(w.scales)
+            assert_close(f64(Y[a:b]), oracle.fwd(fmt, c, s, w.ws2, hbits(X[a:b])), what=f"Y of expert {e}")
+            assert_close(f64(dX[a:b]), oracle.dx(fmt, c, s, w.ws2, hbits(dY[a:b])), what=f"dX of expert {e}")
+
+
+def test_table_ring_reuse_on_the_pair_kernel(h):
+    """As above with experts large enough for the pair kernel, whose tables hold tensor maps:
+    forward and input gradient of changing routings enqueued without a sync."""
+    from paper_2609_04526_gb300 import synth
+    N, K = 1032, 1056
+    wl = synth.custom_moe("ring", NV, PAIR_ROWS, N, K, seed=6)
+    gw, off, X, dY = _setup(wl, wl.linears[0])
+    outs = []
+    for i in range(6):
+        rows = PAIR_ROWS[i:] + PAIR_ROWS[:i]
+        assert _on_pair_kernel(rows, N, K)
+        o = synth.offsets_of(rows)
+        outs.append((o, h.sq_grouped_fwd(gw, o, X), h.sq_grouped_bwd_dx(gw, o, dY)))
+    h.sq_sync()
+    for o, Y, dX in outs:
+        Yd, dXd, _ = _dense_per_expert(h, gw, o, X, dY)
+        h.sq_sync()
+        assert torch.equal(Y, Yd) and torch.equal(dX, dXd)
 
 
 def test_grouped_empty_batches(h):
