@@ -87,6 +87,14 @@ __device__ __forceinline__ void tma_load_2d_elect(uint32_t dst, const CUtensorMa
       : "memory");
 }
 
+// After an abort: waits, with a limit each, for the copies into a ring's slots in flight, of
+// `fills` made so far. All of them (the last may land first); a stage that its decode warps gave
+// up only ends at the limit.
+__device__ __noinline__ void drain_ring(uint64_t *full, int fills, int slots) {
+  for (int i = (fills > slots ? fills - slots : 0); i < fills; ++i)
+    mbar_drain(&full[i % slots], static_cast<uint32_t>(i / slots) & 1u);
+}
+
 // BK: contraction depth of a stage. WARPS: decode warps, which then run the epilogue.
 // GROUPS: see the decode warps. FEAT: output features of a tile; of 64 the MMAs' upper 64
 // rows multiply whatever the shared memory holds, into accumulator lanes that nothing reads.
@@ -167,11 +175,7 @@ __global__ void __launch_bounds__(32 * (WARPS + 3), 16 / WARPS)
         ph ^= 1u;
       }
     }
-    // after an abort: wait, with a limit, for the copies in flight
-    if (*abort_flag) {
-      for (int i = (j > p.slots ? j - p.slots : 0); i < j; ++i)
-        mbar_drain(&cfull[i % p.slots], static_cast<uint32_t>(i / p.slots) & 1u);
-    }
+    if (*abort_flag) drain_ring(cfull, j, p.slots);
     __syncwarp();
   } else if (warp == kTmaWarp) {
     // ------------------------------------------------------ activations
@@ -218,11 +222,7 @@ __global__ void __launch_bounds__(32 * (WARPS + 3), 16 / WARPS)
         ph ^= 1u;
       }
     }
-    // after an abort: wait, with a limit, for the copies in flight (of every stage: the last
-    // one's may land first; a stage that its decode warps gave up only ends at the limit)
-    if (*abort_flag) {
-      for (int i = (it > S ? it - S : 0); i < it; ++i) mbar_drain(&full[i % S], static_cast<uint32_t>(i / S) & 1u);
-    }
+    if (*abort_flag) drain_ring(full, it, S);
     __syncwarp();
   } else if (warp == kMmaWarp) {
     // ------------------------------------------------------ MMA issuer

@@ -39,7 +39,7 @@ def test_aborted_copies_are_waited_for():
     codes (slots) and the activations (stages). A block that ends before a copy lands lets it write
     into the next block's shared memory."""
     src = re.sub(r"\s+", " ", _source("sq_few.cu"))
-    for bar, count, filled in (("cfull", "p.slots", "j"), ("full", "S", "it")):
-        loop = (rf"if \(\*abort_flag\) {{ for \(int i = \({filled} > {count} \? {filled} - {count} : 0\); i < {filled}; \+\+i\) "
-                rf"mbar_drain\(&{bar}\[i % {count}\], static_cast<uint32_t>\(i / {count}\) & 1u\);")
-        assert re.search(loop, src), bar
+    for call in ("drain_ring(cfull, j, p.slots)", "drain_ring(full, it, S)"):
+        assert f"if (*abort_flag) {call};" in src, call
+    assert ("for (int i = (fills > slots ? fills - slots : 0); i < fills; ++i) "
+            "mbar_drain(&full[i % slots], static_cast<uint32_t>(i / slots) & 1u);") in src
