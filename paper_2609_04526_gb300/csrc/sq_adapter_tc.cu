@@ -20,7 +20,8 @@
 // Bound by each CTA's chain of staging, MMAs and drain (two CTAs per SM), so its length in
 // instructions counts: B's staging without divisions, two values split per conversion and
 // the 36 MMAs of a step issued from uniform registers took the kernel from 50 to 41 us for
-// the 128 experts of 768 x 128 blocks at rank 54 (75 MB in and out: 11 us of memory time).
+// the 128 experts of 768 x 128 blocks at rank 54 (75 MB in and out: 11 us of memory time). ncu
+// there: issuing in 39 % of the cycles, tensor pipe 14 %, DRAM 20 %.
 #include "sq_gemm_kernels.cuh"
 
 namespace sqi {

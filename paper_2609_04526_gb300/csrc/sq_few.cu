@@ -21,10 +21,13 @@
 //
 // Measured (forward; before: the pair kernel): 4096 x 4096 at 187 tokens 43 -> 18.5 us, 1024 x
 // 4096 at 2048 tokens 44 -> 25 us, 128 experts of 768 x 2048 with 128 rows each 131 -> 87 us,
-// of 2880 x 2880 with 16 rows each 566 -> 271 us (2.1 TB/s of codes). clock64 traces of one
-// CTA show its pace set by the decode warps' issue slots and by the MMA and TMA warps' own
-// instructions beside them (a barrier test ~110 cycles, a commit ~100, a TMA load ~150), not
-// by the tensor core or the memory: hence the long stages, and one elected lane per warp.
+// of 2880 x 2880 with 16 rows each 566 -> 271 us (2.1 TB/s of codes). Bound by latency: with
+// two CTAs per SM (128 experts of 768 x 2048, 128 rows each) the schedulers issue in 52 % of
+// the cycles forward and 51 % in the input gradient, the tensor pipe is busy for 29 and 24 %,
+// DRAM at 31 and 24 % of its rate, and of the warps waiting most (4.1 and 3.9 per issue) wait on
+// the long scoreboard; a CTA alone issues in 43 %. clock64 traces of one CTA show what a stage's
+// chain consists of (a barrier test ~110 cycles, a commit ~100, a TMA load ~150, beside the
+// decode): hence the long stages, and one elected lane per warp.
 // Codes and activations have a TMA warp each: with one for both a stage of a CTA alone took
 // 0.60 us where it takes 0.54 (4096 x 4096 at 187 tokens 24.7 -> 22.6 us, 4096 x 14336 at 64
 // tokens 71.9 -> 61.6 us; the experts' launches, two CTAs per SM, are unchanged); in tiles of
@@ -305,7 +308,10 @@ __global__ void __launch_bounds__(32 * (WARPS + 3), 16 / WARPS)
     }
     uint32_t sw[C::kAhead];
     auto load = [&](int r) -> uint32_t {  // scale bytes of unit r of the loads' stage
-      uint32_t sc = 0;  // a unit outside the weight is scaled to zeros
+      // Outside the weight byte 0, for NVFP4 a scale of zero. For MXFP4 it is 2^-127, and the
+      // other operand or the store makes up for it: TMA fills the activations with zeros past
+      // the contraction's end, and features past the last are not stored.
+      uint32_t sc = 0;
       if (stages_left > 0 && r * kRowStep < rows_left) {
         const uint8_t *s = sp + static_cast<int64_t>(r * kRowStep) * srow;
         sc = FMT == 0 ? __ldg(reinterpret_cast<const unsigned short *>(s)) : __ldg(s);

@@ -490,9 +490,10 @@ __device__ __forceinline__ uint4 lds128(uint32_t addr) {
 
 // Scale byte(s) covering the 32 weights of one decode unit of the weight whose
 // scale plane starts at `scales`: two E4M3 bytes (blocks of 16) or one E8M0 byte.
-// Units outside the weight read scale 0, so their decoded weights are zero
-// whatever codes the tile holds there (TMA zero fill past the last row, or the
-// next expert's rows in a grouped launch).
+// Units outside the weight read byte 0, whatever codes the tile holds there (TMA zero fill
+// past the last row, or the next expert's rows in a grouped launch). NVFP4 decodes them to
+// zeros; MXFP4's byte 0 is 2^-127, and there the result is right because TMA fills the
+// activations with zeros past the contraction's end and clips stores past the last feature.
 template <int FMT>
 __device__ __forceinline__ uint32_t load_unit_scale(const KParams &p, const uint8_t *scales, int64_t n, int64_t k) {
   if (n >= p.N || k >= p.K) return 0u;
@@ -1360,6 +1361,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg::kThreads, 1
 //  - a unit's place comes from steps and tables in shared memory instead of divisions;
 //  - the TMEM load of a column group runs under the previous group's arithmetic, and the
 //    accumulator is released once its last group is in registers.
+// A 256 x 256 unit takes about 4,200 cycles for 1,024 (128 tokens) or 2,048 (256) of MMAs: ncu
+// shows the schedulers issuing in 63 % of cycles, tensor pipe 27 %, DRAM 36 % and L2 45 % of
+// their rates over 128 experts of 768 x 2048 with 128 rows each; 54, 50, 26 and 49 % over 128 of
+// 2880 x 2880 with 256.
 // With four warps that loaded a group's codes only after its accumulator, a 256-token unit
 // took ~8,600 cycles for 2,048 cycles of MMAs; with eight that fetched a unit ahead, ~5,000.
 // Scale gradients, four warps / eight / now: 128 experts of 2880 x 2880 with 256 rows each

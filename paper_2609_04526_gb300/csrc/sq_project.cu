@@ -253,6 +253,12 @@ __device__ __forceinline__ void project4(float4 L4, const TensorScale &ts, uint3
   }
 }
 
+// One plane per call, or the experts' planes of a grouped call: any address and count (tails
+// of 1 to 15 blocks), where the planes' kernels below need whole vectors and take at most
+// kMaxPlanes planes. Each thread projects 16 consecutive blocks one by one. Against a planes' call
+// with the same single plane, in us with their counters (a memset here): 14336 x 256 blocks
+// NVFP4 projected 9.6 and 8.9, merged 9.5 and 8.3, 14336 x 128 MXFP4 8.2 and 7.2, 8.4 and 6.3;
+// 1024 x 256 6.1 and 6.3, merged with a delta and no count 4.2 and 6.3.
 // Planes of several experts in one launch (PER instantiations): element i belongs
 // to expert i / plane and takes that expert's tensor scale; plane is a multiple
 // of 16, so one 16-element vector never straddles two experts.
@@ -435,8 +441,12 @@ __device__ __forceinline__ void plane_counters(const PlaneTable &t, int j, uint3
 // reads 512 contiguous bytes and each store of bytes writes 128. A thread loads all its
 // latents (and, merging, the old bytes) before it computes and stores any: the byte stores
 // could alias the latent loads as far as the compiler knows, so interleaving them would
-// serialise every float4 on the memory latency. Bound by the memory system at these sizes:
-// the 82 MB of the 8B layer's NVFP4 planes take 21 us projected and 19 us merged (before
+// serialise every float4 on the memory latency. At these sizes a launch is its start, two to
+// four waves of CTAs and load latency: ncu shows the SMs busy for 60 and 66 % of the 20 and
+// 21 us of the 8B layer's NVFP4 planes, the schedulers issuing in 53 and 60 % of those cycles,
+// most waiting warps on their loads, and DRAM at 36 and 42 % of its rate. (Five CTAs per SM
+// cost the NVFP4 projection 20 bytes of spills per thread.)
+// The 82 MB of these planes take 21 us projected and 19 us merged (before
 // project4's short paths 23 and 21), the 41 MB of its MXFP4 planes 12.6 and 12.1 us (18.2 and
 // 17.8). The merge, with the old bytes to hold, is faster with half the float4s per thread;
 // one wave of CTAs that walk the chunks, the next chunk's loads in flight, took 2-3 us more.
@@ -624,11 +634,11 @@ __global__ void __launch_bounds__(kThreads) sq_swap_or_diff_kernel(int64_t count
 // follow expert e - 1's, and grid z (with the contraction chunk for the products)
 // selects the expert; a dense call is the case E = 1.
 // The adapter projection of small ranks and the products for ranks above 128 and of the
-// control are register-tiled fp32 CUDA-core products: a CTA of 256 threads owns a 64 x 64 output tile, its operands staged in shared
-// memory as fp32 (contraction index outermost), and each thread accumulates a 4 x 4 sub-tile
-// (rows ty*4 .. +3, columns tx*4 .. +3), so two 16-byte shared-memory loads feed 16 fused
-// multiply-adds. Every output is summed sequentially over the contraction index, so
-// results do not change between runs.
+// control are register-tiled fp32 CUDA-core products: a CTA of 256 threads owns a 64 x 64
+// output tile, its operands staged in shared memory as fp32 (contraction index outermost), and
+// each thread accumulates a 4 x 4 sub-tile (rows ty*4 .. +3, columns tx*4 .. +3), so two 16-byte
+// shared-memory loads feed 16 fused multiply-adds. Every output is summed sequentially over the
+// contraction index, so results do not change between runs.
 constexpr int kT = 64;   // output tile edge
 constexpr int kTP = 68;  // padded row of a staged operand (16-byte multiple; spreads the transposed stores)
 constexpr int lowrank_smem(int r) { return (kTP + kT) * r * static_cast<int>(sizeof(float)); }  // <= 132 KiB
@@ -742,7 +752,10 @@ __global__ void __launch_bounds__(kThreads) sq_project_lowrank_kernel(
 // per 16 multiply-adds; here four feed 64, taken two blocks at a time by packed
 // multiply-adds (the same rate as single ones, in half the issue slots). B and A are staged
 // as fp32 as they lie: a 16-byte load of B holds four j of a row, one of A four blocks of a
-// j. Ranks above kWideChunk run chunk by chunk on the same accumulators.
+// j. Ranks above kWideChunk run chunk by chunk on the same accumulators. Bound by latency: 12
+// warps per SM (164 registers, 43 KiB) issue in 45 % of the cycles, the most frequent wait is for
+// the previous instruction, and staging, products and projection of a CTA follow each other
+// (ncu, 128 experts of 768 x 128 at rank 54: 60 us, DRAM at 9 %).
 // Measured, against the 4 x 4 tiles: 14336 x 256 blocks at rank 58 20.7 against 26.7 us, 128
 // experts of 768 x 128 at rank 54 65 against 84 us; but 4096 x 256 at rank 16 11.0 against
 // 8.8 us, 1024 x 256 at rank 128 (32 tiles) 22 against 16 us and 128 experts of 2048 x 48 at
